@@ -163,7 +163,7 @@ KERNEL_SOURCES = {
     "int8_split_kernels": ("aloco_sync_kernel.cuh", "aloco_int8.cuh",
                            "aloco_int8.cu"),
     "int8_fused_kernel": ("aloco_sync_kernel.cuh", "aloco_bulk.cuh", "aloco_int8.cuh",
-                          "aloco_int8_fused.cu"),
+                          "aloco_int8_fused.cuh", "aloco_int8_fused.cu", "aloco_int8_fused_odd.cu"),
     "adamw_kernels": ("aloco_sync_kernel.cuh", "aloco_adamw.cu"),
 }
 

@@ -146,6 +146,10 @@ bool int8_fused_fits(int M, aloco_dtype dtype);
 cudaError_t launch_int8_fused(const SyncArgs &a, const Int8Parts &P,
                               aloco_dtype dtype, int sm_count, int max_grid,
                               cudaStream_t stream, int *grid_out);
+// Its instances for parts that start off a multiple of 8 elements.
+cudaError_t launch_int8_fused_odd(const SyncArgs &a, const Int8Parts &P,
+                                  aloco_dtype dtype, int sm_count, int max_grid,
+                                  cudaStream_t stream, int *grid_out);
 cudaError_t launch_int8_encode(const float *x, int8_t *codes, float *scales,
                                float *decoded, bool vec_ok, const Int8Parts &P,
                                int sm_count, cudaStream_t stream);

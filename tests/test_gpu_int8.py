@@ -127,6 +127,35 @@ def test_int8_round_matches_oracle(dt, M, parts_name, form):
     _compare(w, st, corr, orc, g, v, xs)
 
 
+@pytest.mark.parametrize("lead", range(1, 8))
+@pytest.mark.parametrize("dt,M", [("f32", 1), ("f32", 3), ("f32", 8), ("f32", 9),
+                                  ("bf16", 4), ("bf16", 5), ("bf16", 12), ("bf16", 16)])
+def test_blocks_off_a_16_byte_boundary_equal_the_split_form(dt, M, lead):
+    """Parts after one of `lead` elements start off a 16-byte boundary, and
+    the fused form stages their whole blocks as windows: for every offset and
+    for theta and v staged and direct, one and two CTAs per SM and worker
+    groups, bit for bit the split form, with several blocks to a CTA, short
+    blocks between, and a whole last block whose window passes the vector's
+    end."""
+    parts = [lead, 700 * 4096 + 5, 2 * 4096, 3, 4096 - lead - 8 + 16, 4096]
+    w = W.small(sum(parts), M, dt, seed=50 + M)
+    sa, _ = schedule_pair(w.schedule)
+    outs = []
+    for form in ("split", "fused"):
+        g, v, xs = gpu_inputs(w)
+        v.normal_(0, 1e-3, generator=torch.Generator("cuda").manual_seed(M))
+        st = A.sync_int8(g, v, xs, parts=parts, H_sel=w.H_sel[0], H_base=w.H_base,
+                         step=w.start_step, schedule=sa, outer_lr=w.outer_lr,
+                         outer_beta=w.outer_beta, opts=A.default_opts(pass_=FORMS[form]))
+        assert st["status"] == A.OK and st["pass_used"] == FORMS[form]
+        outs.append((st, g, v, xs))
+    (sta, ga, va, xa), (stb, gb, vb, xb) = outs
+    assert torch.equal(ga, gb) and torch.equal(va, vb)
+    assert all(torch.equal(p, q) for p, q in zip(xa, xb))
+    np.testing.assert_allclose(sta["drift"], stb["drift"], rtol=RTOL_STAT)
+    np.testing.assert_allclose(sta["C"], stb["C"], rtol=RTOL_STAT)
+
+
 @pytest.mark.parametrize("dt,M", [("f32", 1), ("f32", 4), ("f32", 7), ("bf16", 2),
                                   ("bf16", 5), ("bf16", 8), ("bf16", 9), ("bf16", 12),
                                   ("bf16", 16), ("f32", 9), ("f32", 12), ("f32", 16)])
