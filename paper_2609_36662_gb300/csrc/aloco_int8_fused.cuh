@@ -546,38 +546,6 @@ __device__ __forceinline__ void outer_step2(const Coef &k, float2 s, float2 g, f
     gp = add2_rn(g, __ffma2_rn(splat2(k.ne_hi), d, __fmul2_rn(splat2(k.ne_lo), d)));
 }
 
-// Warp sums of the P values each lane holds (P a power of two, at most 32)
-// by recursive halving: at each step a lane keeps the half of its values
-// that its lane bit selects and adds the partner's copy of that half; the
-// last steps add across the lanes that share a value.  Lane L returns the
-// warp sum of value L >> (5 - log2 P).  The order is fixed (and a + b = b + a
-// exactly), so every lane holding a value has the same bits.
-template <int P>
-__device__ __forceinline__ float warp_sum_scatter(float (&v)[P]) {
-    static_assert(P >= 1 && P <= 32 && (P & (P - 1)) == 0, "P: a power of two");
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int st = 0; st < 5; ++st) {
-        const int mask = 16 >> st;
-        const int n = P >> st;  // values still held
-        if (n > 1) {
-            const bool up = (lane & mask) != 0;
-#pragma unroll
-            for (int i = 0; i < n / 2; ++i) {
-                const float send = up ? v[i] : v[i + n / 2];
-                const float keep = up ? v[i + n / 2] : v[i];
-                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
-            }
-        } else {
-            v[0] += __shfl_xor_sync(0xffffffffu, v[0], mask);
-        }
-    }
-    return v[0];
-}
-__host__ __device__ constexpr int pow2_at_least(int n) {
-    return n <= 1 ? 1 : 2 * pow2_at_least((n + 1) / 2);
-}
-
 // The workers' energies of a block summed across the warp at once (warp
 // sums by recursive halving, one fp64 row update per worker and block), so
 // no per-worker accumulator stays live through the rest of the block.
@@ -1342,23 +1310,7 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
         if (since_flush > 0) flush_rows(0, EA);
     }
     flush_b();
-    __syncthreads();
-    double e64[M];
-    double b64 = 0.0;
-    if (t == 0) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) b64 += e_w[w][M];
-    }
-#pragma unroll
-    for (int m = 0; m < M; ++m) {
-        double e = 0.0;
-        if (t == 0) {
-#pragma unroll
-            for (int w = 0; w < W; ++w) e += e_w[w][m];
-        }
-        e64[m] = e;
-    }
-    reduce_and_finish<M, W>(a, M, e64, b64, nf);
+    finish_rows<M, W>(a, M, e_w, nf);
 }
 
 namespace {

@@ -9,10 +9,10 @@
 // stores theta', v' and the replica reset from the same registers.
 //
 // Reductions are deterministic: per-thread fp32 partials are promoted to
-// fp64 every kFlush packs, threads are combined by a fixed warp-shuffle tree
-// and a fixed cross-warp order into one fp64 partial per block, and the last
-// block to finish (atomic ticket, no spinning) sums the block partials in
-// block order.  The grid depends only on (M, dtype, n, device), so a round
+// fp64 every kFlush packs, threads are combined in a fixed order within the
+// warp and across warps into one fp64 partial per block, and the last block
+// to finish (atomic ticket, no spinning) sums the block partials in a fixed
+// order.  The grid depends only on (M, dtype, n, device), so a round
 // on the same inputs reproduces its statistics bit for bit.
 #pragma once
 
@@ -173,112 +173,174 @@ struct Pack<true> {
     }
 };
 
-// Block and grid reduction of the per-thread fp64 partials (the block's
-// NW warps all call it).  Each block writes one row of M + 1 partials; the
-// last block to finish (atomic ticket, no spinning) adds the rows in block
-// order and resets the ticket.  The order of every addition is fixed by the
-// grid alone.
-template <int MM, int NW>
-__device__ __forceinline__ void reduce_and_finish(const SyncArgs &a, int M,
-                                                  double (&e64)[MM], double b64,
-                                                  unsigned nf) {
+// Warp sums of the P values each lane holds (P a power of two, at most 32)
+// by recursive halving: at each step a lane keeps the half of its values
+// that its lane bit selects and adds the partner's copy of that half; the
+// last steps add across the lanes that share a value.  Lane L returns the
+// warp sum of value L >> (5 - log2 P).  The order is fixed (and a + b = b + a
+// exactly), so every lane holding a value has the same bits.
+template <int P, typename T>
+__device__ __forceinline__ T warp_sum_scatter(T (&v)[P]) {
+    static_assert(P >= 1 && P <= 32 && (P & (P - 1)) == 0, "P: a power of two");
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int st = 0; st < 5; ++st) {
+        const int mask = 16 >> st;
+        const int n = P >> st;  // values still held
+        if (n > 1) {
+            const bool up = (lane & mask) != 0;
+#pragma unroll
+            for (int i = 0; i < n / 2; ++i) {
+                const T send = up ? v[i] : v[i + n / 2];
+                const T keep = up ? v[i + n / 2] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
+            }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], mask);
+        }
+    }
+    return v[0];
+}
+__host__ __device__ constexpr int pow2_at_least(int n) {
+    return n <= 1 ? 1 : 2 * pow2_at_least((n + 1) / 2);
+}
+// The sum of column `col` over rows 0..n - 1 (n <= 32), in every lane.
+template <int COLS>
+__device__ __forceinline__ double column_sum(const double (*rows)[COLS], int n, int col) {
+    const int lane = threadIdx.x & 31;
+    double v = lane < n ? rows[lane][col] : 0.0;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
+}
+
+// Grid reduction of the block's fp64 rows: warp w wrote rows[w][m] for m < M
+// and rows[w][MM] (sum S^2); the block's NW warps all call it.  Each block
+// writes one row of M + 1 partials; the last block to finish (atomic ticket,
+// no spinning) adds the rows in a fixed order, resets the ticket and
+// publishes the totals.  The order of every addition is fixed by the grid.
+// Latency-bound, on a part whose SM adds two doubles a clock: a warp-wide
+// fp64 add holds the pipe for 16 clocks, so the work is laid out for few of
+// them.  One warp folds a column (five adds); the grid's rows are read as k
+// interleaved slices, one thread per slice and column, which keeps eight
+// loads in flight and the additions of different columns in one instruction.
+// The host page is written by the threads that hold the totals, together.
+template <int MM, int NW, int S>
+__device__ __forceinline__ void finish_rows(const SyncArgs &a, int M, double (&rows)[S][MM + 1],
+                                            unsigned nf) {
+    static_assert(S >= NW && S <= 32, "a warp folds a column of rows");
     constexpr int kThreads = NW * 32;
-    __shared__ double sh[NW][MM + 1];
     __shared__ unsigned long long shnf[NW];
     __shared__ bool s_last;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-
-    unsigned long long nfl = nf;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-        for (int m = 0; m < MM; ++m)
-            e64[m] += __shfl_down_sync(0xffffffffu, e64[m], off);
-        b64 += __shfl_down_sync(0xffffffffu, b64, off);
-        nfl += __shfl_down_sync(0xffffffffu, nfl, off);
-    }
-    if (lane == 0) {
-#pragma unroll
-        for (int m = 0; m < MM; ++m) sh[warp][m] = e64[m];
-        sh[warp][MM] = b64;
-        shnf[warp] = nfl;
-    }
-    __syncthreads();
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int np = M + 1;  // values per block: M energies + sum S^2
-    if (threadIdx.x < np) {
-        const int col = threadIdx.x < M ? threadIdx.x : MM;
-        double t = 0.0;
+    auto slot = [&](int p) { return p < M ? p : MM; };
+    auto warp_sum = [](unsigned long long v) {
 #pragma unroll
-        for (int w = 0; w < NW; ++w) t += sh[w][col];
-        a.partials[(int64_t)blockIdx.x * np + threadIdx.x] = t;
-    }
-    if (threadIdx.x == kThreads - 1) {
-        unsigned long long t = 0;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) t += shnf[w];
-        a.nf_partials[blockIdx.x] = t;
-    }
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+        return v;
+    };
 
-    __threadfence();
+    const unsigned long long nfl = warp_sum(nf);
+    if (lane == 0) shnf[warp] = nfl;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    for (int p = warp; p < np; p += NW) {
+        const double v = column_sum(rows, NW, slot(p));
+        if (lane == 0) a.partials[(int64_t)blockIdx.x * np + p] = v;
+    }
+    if (t == kThreads - 1) {
+        unsigned long long n = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) n += shnf[w];
+        a.nf_partials[blockIdx.x] = n;
+    }
+    // thread 0's fence after the barrier orders the whole block's writes
+    // (the outputs too) before its ticket
+    __syncthreads();
+    if (t == 0) {
+        __threadfence();
         const unsigned prev = atomicAdd(a.ticket, 1u);
         s_last = (prev == gridDim.x - 1);
+        __threadfence();
     }
     __syncthreads();
     if (!s_last) return;
-    __threadfence();
 
-    double acc[MM + 1];
-#pragma unroll
-    for (int p = 0; p <= MM; ++p) acc[p] = 0.0;
+    const int grid = (int)gridDim.x;
+    const int k = kThreads / np < S ? kThreads / np : S;  // slices of rows
+    const int r = t / np, p = t - r * np;
     unsigned long long nacc = 0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += kThreads) {
-        const double *row = a.partials + (int64_t)b * np;
+    for (int b = t; b < grid; b += kThreads) nacc += __ldcg(a.nf_partials + b);
+    if (r < k) {
+        double acc = 0.0;
+        for (int b0 = r; b0 < grid; b0 += 8 * k) {
+            double q[8];
 #pragma unroll
-        for (int p = 0; p <= MM; ++p)
-            if (p < np) acc[p] += __ldcg(row + p);
-        nacc += __ldcg(a.nf_partials + b);
+            for (int u = 0; u < 8; ++u) {
+                const int b = b0 + u * k;
+                q[u] = b < grid ? __ldcg(a.partials + (int64_t)b * np + p) : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) acc += q[u];
+        }
+        rows[r][slot(p)] = acc;
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-        for (int p = 0; p <= MM; ++p)
-            acc[p] += __shfl_down_sync(0xffffffffu, acc[p], off);
-        nacc += __shfl_down_sync(0xffffffffu, nacc, off);
-    }
-    __syncthreads();  // sh is reused
-    if (lane == 0) {
-#pragma unroll
-        for (int p = 0; p <= MM; ++p) sh[warp][p] = acc[p];
-        shnf[warp] = nacc;
-    }
+    nacc = warp_sum(nacc);
+    if (lane == 0) shnf[warp] = nacc;
     __syncthreads();
-    if (threadIdx.x < np) {
-        double t = 0.0;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) t += sh[w][threadIdx.x];
-        a.totals[threadIdx.x] = t;
+    volatile double *out = a.stats_out;
+    for (int c = warp; c < np; c += NW) {
+        const double v = column_sum(rows, k, slot(c));
+        if (lane == 0) {
+            a.totals[c] = v;
+            if (out) out[c] = v;
+        }
     }
-    if (threadIdx.x == kThreads - 1) {
-        unsigned long long t = 0;
+    if (t == kThreads - 1) {
+        unsigned long long n = 0;
 #pragma unroll
-        for (int w = 0; w < NW; ++w) t += shnf[w];
-        *a.nf_total = t;
+        for (int w = 0; w < NW; ++w) n += shnf[w];
+        *a.nf_total = n;
         *a.ticket = 0u;  // ready for the next launch
-    }
-    if (a.stats_out) {
-        // publish the totals block to the host, then the round's number
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            volatile double *out = a.stats_out;
-            for (int p = 0; p < np; ++p) out[p] = __ldcg(a.totals + p);
-            out[kNfSlot] = __longlong_as_double((long long)__ldcg(a.nf_total));
+        if (out) {
+            out[kNfSlot] = __longlong_as_double((long long)n);
             out[kErrorSlot] = __ldcg(a.totals + kErrorSlot);
+        }
+    }
+    if (out) {
+        // the totals are written: the round's number follows, behind a fence
+        // that orders the block's writes to the page before it
+        __syncthreads();
+        if (t == 0) {
             __threadfence_system();
             reinterpret_cast<volatile unsigned long long *>(a.stats_out)[kSeqSlot] = a.seq;
         }
     }
+}
+
+// The same from per-thread fp64 partials, folded across each warp first:
+// the energies by recursive halving (about MM adds a warp instead of 5 MM).
+// Against shuffle trees over every value in every thread, serial folds in one
+// thread and a serial publish: 2^20 parameters x 4 fp32 workers 20.0 -> 15.1
+// us (the kernel, ncu), 6e6 x 32 bf16 190 -> 166 us; the fused INT8 kernel, 1024
+// threads a block, 2e7 x 16 bf16 385 -> 300 us, 2e7 x 8 fp32 330 -> 283 us.  S bounds the rows where shared memory is short.
+template <int MM, int NW, int S = 32>
+__device__ __forceinline__ void reduce_and_finish(const SyncArgs &a, int M,
+                                                  double (&e64)[MM], double b64,
+                                                  unsigned nf) {
+    constexpr int P = pow2_at_least(MM);
+    __shared__ double rows[S][MM + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double v[P];
+#pragma unroll
+    for (int m = 0; m < P; ++m) v[m] = m < MM ? e64[m < MM ? m : 0] : 0.0;
+    const double e = warp_sum_scatter<P>(v);
+    const int w = lane / (32 / P);
+    if (lane % (32 / P) == 0 && w < MM) rows[warp][w] = e;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) b64 += __shfl_down_sync(0xffffffffu, b64, off);
+    if (lane == 0) rows[warp][MM] = b64;
+    finish_rows<MM, NW>(a, M, rows, nf);
 }
 
 // Minimum resident blocks per SM the register allocator must allow (it

@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(T, (tile_ctas<M, BF16, T>()))
     constexpr uint32_t kStage = 2 * kF + M * kX;
     constexpr uint32_t kOut = (uint32_t)tile_out_bytes<BF16, T, GV>();
 
-    __shared__ double e_w[W][M];
+    __shared__ double e_w[W][M + 1];  // [warp][worker energies, then sum S^2]
     __shared__ __align__(8) unsigned long long full_bar[NS];
     extern __shared__ __align__(128) unsigned char smem[];
 
@@ -348,18 +348,10 @@ __global__ void __launch_bounds__(T, (tile_ctas<M, BF16, T>()))
     if (t == 0) bulk_wait_all();
     flush();
     b64 += (double)b32;
-    __syncthreads();
-    double e64[M];
 #pragma unroll
-    for (int m = 0; m < M; ++m) {
-        double e = 0.0;
-        if (t == 0) {
-#pragma unroll
-            for (int w = 0; w < W; ++w) e += e_w[w][m];
-        }
-        e64[m] = e;
-    }
-    reduce_and_finish<M, W>(a, M, e64, b64, nf);
+    for (int off = 16; off > 0; off >>= 1) b64 += __shfl_down_sync(0xffffffffu, b64, off);
+    if (lane == 0) e_w[warp][M] = b64;
+    finish_rows<M, W>(a, M, e_w, nf);
 }
 
 namespace {

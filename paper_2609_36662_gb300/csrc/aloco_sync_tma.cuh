@@ -249,7 +249,8 @@ __global__ void __launch_bounds__(kTmaThreads, 1)
         }
     }
     flush();
-    reduce_and_finish<M, kTmaThreads / 32>(a, M, e64, b64, nf);
+    // the ring leaves room for one row of totals a warp
+    reduce_and_finish<M, kTmaThreads / 32, kTmaThreads / 32>(a, M, e64, b64, nf);
 }
 
 // Largest ring that fits the shared-memory budget, 2..kTmaMaxStages stages.
