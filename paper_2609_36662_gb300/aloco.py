@@ -6,8 +6,10 @@ raises on first use; there is no fallback path.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
+import struct
 from dataclasses import dataclass
 from typing import Optional, Sequence
 
@@ -109,11 +111,21 @@ class Stats(ctypes.Structure):
                 ("kernel_ms", ctypes.c_float), ("pass_used", ctypes.c_int32)]
 
     def as_dict(self):
-        return {"D": self.D, "C": self.C, "mean_sq_norm": self.mean_sq_norm,
-                "drift": list(self.drift[:self.M]),
-                "corr": self.corr.as_dict(), "nonfinite": self.nonfinite,
-                "M": self.M, "grid": self.grid, "kernel_ms": self.kernel_ms,
-                "pass_used": self.pass_used}
+        # one unpack of the struct: reading the fields one by one through
+        # ctypes costs several microseconds a call
+        f = _STATS.unpack_from(self)
+        M = f[_AT_M]
+        return {"D": f[0], "C": f[1], "mean_sq_norm": f[2],
+                "drift": list(f[3:3 + M]),
+                "corr": dict(zip(_CORR_NAMES, f[3 + MAX_WORKERS:_AT_M - 1])),
+                "nonfinite": f[_AT_M - 1], "M": M, "grid": f[_AT_M + 1],
+                "kernel_ms": f[_AT_M + 2], "pass_used": f[_AT_M + 3]}
+
+
+_CORR_NAMES = tuple(n for n, _ in Correction._fields_)
+_STATS = struct.Struct("=%ddqiifi" % (3 + MAX_WORKERS + len(_CORR_NAMES)))
+_AT_M = 3 + MAX_WORKERS + len(_CORR_NAMES) + 1  # index of M in the unpacked fields
+assert _STATS.size == ctypes.sizeof(Stats)
 
 
 class Partials(ctypes.Structure):
@@ -309,6 +321,39 @@ def correction(schedule: Schedule, step: int, H_sel: int, H_base: int,
     return out
 
 
+def _stream_of(stream, device) -> int:
+    """The raw handle of `stream`, or of the device's current stream."""
+    if stream is not None:
+        return stream.cuda_stream
+    import torch
+    if device.index is None:
+        return torch.cuda.current_stream(device).cuda_stream
+    return torch._C._cuda_getCurrentRawStream(device.index)
+
+
+class _NoSwitch:
+    def __enter__(self):
+        pass
+
+    def __exit__(self, *exc):
+        return False
+
+
+_NO_SWITCH = _NoSwitch()
+
+
+def _on_device(device):
+    """A context with `device` current; nothing to do where it already is."""
+    import torch
+    if torch.cuda.current_device() == device.index:
+        return _NO_SWITCH
+    return torch.cuda.device(device)
+
+
+def _pointers(tensors):
+    return (ctypes.c_void_p * len(tensors))(*[t.data_ptr() for t in tensors])
+
+
 def sync_ptrs(g_ptr: int, v_ptr: int, x_ptrs: Sequence[int], N: int,
               dtype: int, H_sel: int, H_base: int, step: int,
               schedule: Schedule, outer_lr: float, outer_beta: float,
@@ -341,6 +386,32 @@ def sync(global_, momentum, locals_, *, H_sel: int, H_base: int, step: int,
     current torch stream).  noalloc=True calls aloco_sync_noalloc, the entry
     point that allocates nothing (its scratch is a static device array)."""
     import torch
+    N = global_.numel()
+    rdt = locals_[0].dtype if locals_ else None
+    if not (global_.dtype == momentum.dtype == torch.float32
+            and momentum.numel() == N and rdt in (torch.float32, torch.bfloat16)
+            and all([t.is_cuda and t.is_contiguous() for t in (global_, momentum)])
+            and all([x.dtype == rdt and x.numel() == N and x.is_cuda
+                     and x.is_contiguous() for x in locals_])):
+        _refuse_round(global_, momentum, locals_)
+    dtype = F32 if rdt == torch.float32 else BF16
+    if opts is None:
+        opts = default_opts()
+    device = global_.device
+    opts.stream = _stream_of(stream, device)
+    with _on_device(device):
+        rc, st = sync_ptrs(global_.data_ptr(), momentum.data_ptr(),
+                           [x.data_ptr() for x in locals_], N, dtype, H_sel,
+                           H_base, step, schedule, outer_lr, outer_beta, opts,
+                           raise_on_error, noalloc)
+    out = st.as_dict()
+    out["status"] = rc
+    return out
+
+
+def _refuse_round(global_, momentum, locals_):
+    """Raise what is wrong with sync()'s tensors."""
+    import torch
     if global_.dtype != torch.float32 or momentum.dtype != torch.float32:
         raise TypeError("global and momentum must be float32")
     N = global_.numel()
@@ -351,26 +422,9 @@ def sync(global_, momentum, locals_, *, H_sel: int, H_base: int, step: int,
     rdt = locals_[0].dtype
     if any(x.dtype != rdt for x in locals_):
         raise TypeError("replicas must share one dtype")
-    if rdt == torch.float32:
-        dtype = F32
-    elif rdt == torch.bfloat16:
-        dtype = BF16
-    else:
+    if rdt not in (torch.float32, torch.bfloat16):
         raise TypeError(f"unsupported replica dtype {rdt}")
-    for t in (global_, momentum, *locals_):
-        if not t.is_cuda or not t.is_contiguous():
-            raise ValueError("buffers must be contiguous CUDA tensors")
-    if opts is None:
-        opts = default_opts()
-    s = stream if stream is not None else torch.cuda.current_stream(
-        global_.device)
-    opts.stream = s.cuda_stream
-    with torch.cuda.device(global_.device):
-        rc, st = sync_ptrs(global_.data_ptr(), momentum.data_ptr(),
-                           [x.data_ptr() for x in locals_], N, dtype, H_sel,
-                           H_base, step, schedule, outer_lr, outer_beta, opts,
-                           raise_on_error, noalloc)
-    return st.as_dict() | {"status": rc}
+    raise ValueError("buffers must be contiguous CUDA tensors")
 
 
 def shutdown():
@@ -397,9 +451,8 @@ def sync_shard(global_, momentum, locals_, *, H_sel: int, H_base: int,
     elements), in place: aloco_sync_shard, or aloco_sync_int8_shard with
     int8=True (parts: the shard's tensor parts).  Returns (status,
     Partials)."""
-    import torch
     N = global_.numel()
-    if momentum.numel() != N or any(x.numel() != N for x in locals_):
+    if momentum.numel() != N or any([x.numel() != N for x in locals_]):
         raise ValueError("all buffers must have the same number of elements")
     for t in (global_, momentum, *locals_):
         if not t.is_cuda or not t.is_contiguous():
@@ -407,13 +460,11 @@ def sync_shard(global_, momentum, locals_, *, H_sel: int, H_base: int,
     dtype = _replica_dtype_code(locals_[0])
     if opts is None:
         opts = default_opts()
-    s = stream if stream is not None else torch.cuda.current_stream(
-        global_.device)
-    opts.stream = s.cuda_stream
+    opts.stream = _stream_of(stream, global_.device)
     M = len(locals_)
-    ptrs = (ctypes.c_void_p * M)(*[x.data_ptr() for x in locals_])
+    ptrs = _pointers(locals_)
     out = Partials()
-    with torch.cuda.device(global_.device):
+    with _on_device(global_.device):
         if int8:
             arr, n = _parts_array(parts)
             rc = load().aloco_sync_int8_shard(
@@ -496,8 +547,8 @@ class Controller:
 def _parts_array(parts):
     if parts is None:
         return None, 0
-    arr = (ctypes.c_int64 * len(parts))(*[int(p) for p in parts])
-    return arr, len(parts)
+    buf = array.array("q", [int(p) for p in parts])
+    return (ctypes.c_int64 * len(parts)).from_buffer(buf), len(parts)
 
 
 def int8_num_blocks(parts) -> int:
@@ -525,13 +576,12 @@ def int8_encode(x, parts=None, want_decoded=True, stream=None):
     codes = torch.empty(N, dtype=torch.int8, device=x.device)
     scales = torch.empty(nb, dtype=torch.float32, device=x.device)
     dec = torch.empty_like(x) if want_decoded else None
-    s = stream if stream is not None else torch.cuda.current_stream(x.device)
     arr, n = _parts_array(parts)
-    with torch.cuda.device(x.device):
+    with _on_device(x.device):
         rc = load().aloco_int8_encode(x.data_ptr(), N, arr, n,
                                       codes.data_ptr(), scales.data_ptr(),
                                       dec.data_ptr() if dec is not None
-                                      else None, s.cuda_stream)
+                                      else None, _stream_of(stream, x.device))
     if rc != OK:
         raise AlocoError(rc, last_error())
     return codes, scales, dec
@@ -541,12 +591,11 @@ def int8_decode(codes, scales, parts=None, stream=None):
     import torch
     N = codes.numel()
     out = torch.empty(N, dtype=torch.float32, device=codes.device)
-    s = stream if stream is not None else torch.cuda.current_stream(
-        codes.device)
     arr, n = _parts_array(parts)
-    with torch.cuda.device(codes.device):
+    with _on_device(codes.device):
         rc = load().aloco_int8_decode(codes.data_ptr(), scales.data_ptr(), N,
-                                      arr, n, out.data_ptr(), s.cuda_stream)
+                                      arr, n, out.data_ptr(),
+                                      _stream_of(stream, codes.device))
     if rc != OK:
         raise AlocoError(rc, last_error())
     return out
@@ -589,14 +638,12 @@ def sync_int8(global_, momentum, locals_, *, parts=None, H_sel: int,
     dtype = F32 if rdt == torch.float32 else BF16
     if opts is None:
         opts = default_opts()
-    s = stream if stream is not None else torch.cuda.current_stream(
-        global_.device)
-    opts.stream = s.cuda_stream
+    opts.stream = _stream_of(stream, global_.device)
     M = len(locals_)
-    ptrs = (ctypes.c_void_p * M)(*[x.data_ptr() for x in locals_])
+    ptrs = _pointers(locals_)
     arr, n = _parts_array(parts)
     st = Stats()
-    with torch.cuda.device(global_.device):
+    with _on_device(global_.device):
         rc = load().aloco_sync_int8(global_.data_ptr(), momentum.data_ptr(),
                                     ptrs, N, M, dtype, H_sel, H_base, step,
                                     ctypes.byref(schedule), outer_lr,
@@ -604,7 +651,9 @@ def sync_int8(global_, momentum, locals_, *, parts=None, H_sel: int,
                                     ctypes.byref(st))
     if raise_on_error and rc not in (OK, ERR_NONFINITE):
         raise AlocoError(rc, last_error())
-    return st.as_dict() | {"status": rc}
+    out = st.as_dict()
+    out["status"] = rc
+    return out
 
 
 # ----------------------------------------------------- inner AdamW (Sec. 2)
@@ -639,14 +688,10 @@ def adamw_step(params, grads, exp_avg, exp_avg_sq, cfg: AdamwCfg,
     gdt = F32 if grads[0].dtype == torch.float32 else BF16
     if opts is None:
         opts = default_opts()
-    s = stream if stream is not None else torch.cuda.current_stream(
-        params[0].device)
-    opts.stream = s.cuda_stream
-
-    def arr(ts):
-        return (ctypes.c_void_p * M)(*[t.data_ptr() for t in ts])
+    opts.stream = _stream_of(stream, params[0].device)
+    arr = _pointers
     st = AdamwStats() if want_stats else None
-    with torch.cuda.device(params[0].device):
+    with _on_device(params[0].device):
         if grad_norms is None:
             rc = load().aloco_adamw_step(arr(params), arr(grads), arr(exp_avg),
                                          arr(exp_avg_sq), N, M, pdt, gdt,

@@ -75,26 +75,40 @@ double lr_at(const aloco_schedule_t &s, int64_t k) {
 // sum_{h=1..H} lr(t0 + h - 1), Neumaier-compensated.  Segments where the
 // rate is constant (constant schedule, the tail after total_steps) are
 // summed as a product.
-double lr_mass(const aloco_schedule_t &s, int64_t t0, int64_t H) {
-    if (H <= 0) return 0.0;
-    if (s.kind == ALOCO_SCHED_CONSTANT) return (double)H * s.peak_lr;
-    const int64_t end = t0 + H;  // exclusive
-    const int64_t vary_end = end < s.total_steps ? end : s.total_steps;
+struct MassSum {
     double sum = 0.0, comp = 0.0;
-    for (int64_t k = t0; k < vary_end; ++k) {
-        const double x = lr_at(s, k);
+    void add(double x) {
         const double t = sum + x;
         comp += std::fabs(sum) >= std::fabs(x) ? (sum - t) + x : (x - t) + sum;
         sum = t;
     }
-    const int64_t tail_begin = t0 > s.total_steps ? t0 : s.total_steps;
-    if (end > tail_begin) {
-        const double x = (double)(end - tail_begin) * s.final_lr;
-        const double t = sum + x;
-        comp += std::fabs(sum) >= std::fabs(x) ? (sum - t) + x : (x - t) + sum;
-        sum = t;
+};
+
+// The sums of two horizons that start at the same step, H[0] <= H[1]: the
+// rates of the shorter one are a prefix of the longer one's, so each rate is
+// evaluated once (the cosines are most of the host's arithmetic in a round).
+void lr_mass2(const aloco_schedule_t &s, int64_t t0, const int64_t (&H)[2], double (&out)[2]) {
+    MassSum m;
+    int64_t k = t0;
+    for (int i = 0; i < 2; ++i) {
+        if (H[i] <= 0 || s.kind == ALOCO_SCHED_CONSTANT) {
+            out[i] = H[i] <= 0 ? 0.0 : (double)H[i] * s.peak_lr;
+            continue;
+        }
+        const int64_t end = t0 + H[i];  // exclusive
+        const int64_t vary_end = end < s.total_steps ? end : s.total_steps;
+        for (; k < vary_end; ++k) m.add(lr_at(s, k));
+        MassSum whole = m;
+        const int64_t tail_begin = t0 > s.total_steps ? t0 : s.total_steps;
+        if (end > tail_begin) whole.add((double)(end - tail_begin) * s.final_lr);
+        out[i] = whole.sum + whole.comp;
     }
-    return sum + comp;
+}
+
+double lr_mass(const aloco_schedule_t &s, int64_t t0, int64_t H) {
+    double out[2];
+    lr_mass2(s, t0, {H, H}, out);
+    return out[0];
 }
 
 // ----------------------------------------------------------- correction
@@ -132,8 +146,10 @@ int correction_impl(const aloco_schedule_t *sched, int64_t step,
 
     aloco_correction_t c;
     // Eq. app-outer-correction-lr-masses: both previews start at s_t = step.
-    c.lam_sel = lr_mass(*sched, step, H_sel);
-    c.lam_base = lr_mass(*sched, step, H_base);
+    double mass[2];
+    lr_mass2(*sched, step, {std::min(H_sel, H_base), std::max(H_sel, H_base)}, mass);
+    c.lam_sel = mass[H_sel > H_base];
+    c.lam_base = mass[H_base > H_sel];
     // Eq. app-outer-correction-ratios.
     c.rho_unc = c.lam_sel / (c.lam_base + o.eps);
     c.rho = std::fmax(c.rho_unc, 1.0);
@@ -274,14 +290,15 @@ int ensure_ready(Workspace *ws, int device) {
 // SyncArgs::stats_out).  The last block publishes after every block's
 // outputs are written, so on return the outputs are complete, and work
 // queued later on the stream runs after the kernel.  The stream is polled
-// every few hundred reads: a launch that fails or ends without publishing
-// returns an error instead of waiting on.
+// every few thousand reads (some microseconds; a query takes about one, in
+// which the flag is not seen): a launch that fails or ends without
+// publishing returns an error instead of waiting on.
 int wait_published(const double *page, unsigned long long seq, cudaStream_t stream) {
     const volatile unsigned long long *flag =
         reinterpret_cast<const volatile unsigned long long *>(page + aloco::kSeqSlot);
     for (unsigned it = 1;; ++it) {
         if (*flag == seq) break;
-        if ((it & 255) == 0) {
+        if ((it & 4095) == 0) {
             const cudaError_t q = cudaStreamQuery(stream);
             if (q == cudaErrorNotReady) continue;
             if (q != cudaSuccess) return cuda_fail(q, "round");
@@ -379,19 +396,25 @@ int report_error(int code, const char *msg) { return fail(code, "%s", msg); }
 
 // The buffer must be device (or managed) memory of `device`, and when the
 // driver can tell, [p, p + bytes) must lie inside one allocation.
-int check_buffer(const void *p, size_t bytes, int device, const char *name) {
+int check_buffer(const void *p, size_t bytes, int device, const char *base, int index) {
     cudaPointerAttributes at;
+    const auto name_of = [&](char (&buf)[48]) -> const char * {
+        if (index < 0) return base;
+        snprintf(buf, sizeof buf, "%s[%d]", base, index);
+        return buf;
+    };
+    char name_buf[48];
     cudaError_t e = cudaPointerGetAttributes(&at, p);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        return fail(ALOCO_ERR_ARG, "%s: not a CUDA pointer (%s)", name,
+        return fail(ALOCO_ERR_ARG, "%s: not a CUDA pointer (%s)", name_of(name_buf),
                     cudaGetErrorString(e));
     }
     if (at.type != cudaMemoryTypeDevice && at.type != cudaMemoryTypeManaged)
-        return fail(ALOCO_ERR_ARG, "%s: not device memory", name);
+        return fail(ALOCO_ERR_ARG, "%s: not device memory", name_of(name_buf));
     if (at.type == cudaMemoryTypeDevice && at.device != device)
         return fail(ALOCO_ERR_ARG, "%s: lives on device %d, current device is %d",
-                    name, at.device, device);
+                    name_of(name_buf), at.device, device);
     if (GetAddressRangeFn fn = address_range_fn()) {
         CUdeviceptr base = 0;
         size_t size = 0;
@@ -400,7 +423,7 @@ int check_buffer(const void *p, size_t bytes, int device, const char *name) {
                 return fail(ALOCO_ERR_ARG,
                             "%s: %zu bytes from %p run past the end of its "
                             "allocation (%zu bytes at %p)",
-                            name, bytes, p, size, (void *)base);
+                            name_of(name_buf), bytes, p, size, (void *)base);
         }
     }
     return ALOCO_OK;
@@ -612,9 +635,7 @@ int sync_impl(float *global, float *momentum, void *const *locals, size_t N,
     if ((rc = check_buffer(global, N * 4, device, "global")) != ALOCO_OK) return rc;
     if ((rc = check_buffer(momentum, N * 4, device, "momentum")) != ALOCO_OK) return rc;
     for (int m = 0; m < M; ++m) {
-        char name[32];
-        snprintf(name, sizeof name, "locals[%d]", m);
-        if ((rc = check_buffer(locals[m], N * rsz, device, name)) != ALOCO_OK)
+        if ((rc = check_buffer(locals[m], N * rsz, device, "locals", m)) != ALOCO_OK)
             return rc;
     }
 
@@ -1333,15 +1354,11 @@ static int adamw_impl(void *const *params, const void *const *grads,
     int rc = ensure_ready(ws, device);
     if (rc != ALOCO_OK) return rc;
     for (int m = 0; m < M; ++m) {
-        char name[40];
-        snprintf(name, sizeof name, "params[%d]", m);
-        if ((rc = check_buffer(params[m], N * psz, device, name)) != ALOCO_OK) return rc;
-        snprintf(name, sizeof name, "grads[%d]", m);
-        if ((rc = check_buffer(grads[m], N * gsz, device, name)) != ALOCO_OK) return rc;
-        snprintf(name, sizeof name, "exp_avg[%d]", m);
-        if ((rc = check_buffer(exp_avg[m], N * 4, device, name)) != ALOCO_OK) return rc;
-        snprintf(name, sizeof name, "exp_avg_sq[%d]", m);
-        if ((rc = check_buffer(exp_avg_sq[m], N * 4, device, name)) != ALOCO_OK) return rc;
+        if ((rc = check_buffer(params[m], N * psz, device, "params", m)) != ALOCO_OK ||
+            (rc = check_buffer(grads[m], N * gsz, device, "grads", m)) != ALOCO_OK ||
+            (rc = check_buffer(exp_avg[m], N * 4, device, "exp_avg", m)) != ALOCO_OK ||
+            (rc = check_buffer(exp_avg_sq[m], N * 4, device, "exp_avg_sq", m)) != ALOCO_OK)
+            return rc;
     }
 
     aloco::AdamArgs a;

@@ -187,7 +187,8 @@ cudaError_t launch_adamw(const AdamArgs &a, aloco_dtype param_dtype,
 
 // Host helpers shared by the entry points (aloco_host.cpp).
 int report_error(int code, const char *msg);
-int check_buffer(const void *p, size_t bytes, int device, const char *name);
+// (base, index >= 0: the message names base[index])
+int check_buffer(const void *p, size_t bytes, int device, const char *base, int index = -1);
 void fill_default_opts(aloco_opts_t *o);
 void split_coef(double x, float *hi, float *lo);
 // b_scale converts the last total into ||Dbar||^2: 1/M^2 when the pass

@@ -174,9 +174,7 @@ extern "C" int aloco_sync_noalloc(float *global, float *momentum,
     if ((rc = aloco::check_buffer(momentum, N * 4, device, "momentum")) != ALOCO_OK)
         return rc;
     for (int m = 0; m < M; ++m) {
-        char name[32];
-        snprintf(name, sizeof name, "locals[%d]", m);
-        if ((rc = aloco::check_buffer(locals[m], N * rsz, device, name)) != ALOCO_OK)
+        if ((rc = aloco::check_buffer(locals[m], N * rsz, device, "locals", m)) != ALOCO_OK)
             return rc;
     }
 
