@@ -444,6 +444,34 @@ void fill_default_opts(aloco_opts_t *o) {
     o->wait = ALOCO_WAIT_SPIN;
 }
 
+void set_buffers(SyncArgs *a, float *global, float *momentum, void *const *locals,
+                 size_t N, int M, aloco_dtype dtype) {
+    const size_t rsz = dtype == ALOCO_F32 ? 4 : 2;
+    const size_t pack = (size_t)pack_elems(dtype);
+    // elements from a buffer's start to its next 16-byte boundary, by the
+    // replicas; theta and v repeat theirs every four elements
+    const auto to_boundary = [](const void *p, size_t size) {
+        return (size_t)((16 - ((uintptr_t)p & 15)) & 15) / size;
+    };
+    size_t head = to_boundary(locals[0], rsz);
+    bool same = to_boundary(global, 4) == head % 4 && to_boundary(momentum, 4) == head % 4;
+    for (int m = 1; m < M; ++m) same = same && to_boundary(locals[m], rsz) == head;
+    if (!same || head >= N) head = 0;
+    a->head = (int)head;
+    a->g = global + head;
+    a->v = momentum + head;
+    for (int m = 0; m < M; ++m) a->x[m] = static_cast<char *>(locals[m]) + head * rsz;
+    a->n = (int64_t)(N - head);
+    a->nvec = same ? (int64_t)((N - head) / pack) : 0;
+    if (a->nvec == 0 && head > 0) {  // too short for a pack: elements only
+        a->head = 0;
+        a->g = global;
+        a->v = momentum;
+        for (int m = 0; m < M; ++m) a->x[m] = locals[m];
+        a->n = (int64_t)N;
+    }
+}
+
 // x ~= hi + lo with hi = fl32(x), lo = fl32(x - hi).
 void split_coef(double x, float *hi, float *lo) {
     *hi = (float)x;
@@ -642,16 +670,9 @@ int sync_impl(float *global, float *momentum, void *const *locals, size_t N,
     // ------------------------------------------------------- launch
     aloco::SyncArgs a;
     std::memset(&a, 0, sizeof a);
-    a.g = global;
-    a.v = momentum;
-    uintptr_t align_or = (uintptr_t)global | (uintptr_t)momentum;
-    for (int m = 0; m < M; ++m) {
-        a.x[m] = locals[m];
-        align_or |= (uintptr_t)locals[m];
-    }
-    const int pack = aloco::pack_elems(dtype);
-    a.n = (int64_t)N;
-    a.nvec = (align_or & 15) == 0 ? (int64_t)(N / pack) : 0;
+    aloco::set_buffers(&a, global, momentum, locals, N, M, dtype);
+    // codec blocks count from the pointers too
+    for (int p = 0; int8 && p <= P.n_parts; ++p) P.off[p] -= a.head;
     // plain pass: Dtil = (inv/M) sum_m Delta_m; INT8 pass: Dtil = inv * mean
     split_coef(int8 ? corr.inv_norm : corr.inv_norm / (double)M, &a.c_hi, &a.c_lo);
     split_coef(corr.mu_t, &a.mu_hi, &a.mu_lo);
@@ -665,8 +686,10 @@ int sync_impl(float *global, float *momentum, void *const *locals, size_t N,
 
     const int64_t work = a.nvec > 0 ? a.nvec : a.n;
     aloco::LaunchPlan plan;
-    const bool tile = !int8 && aloco::use_tile(o.pass, M, dtype, a.n, a.nvec);
-    const bool tma = !int8 && !tile && aloco::use_tma(o.pass, M, dtype, a.nvec);
+    // the staged passes take aligned buffers; the register pass serves a head
+    const int64_t staged = a.head == 0 ? a.nvec : 0;
+    const bool tile = !int8 && aloco::use_tile(o.pass, M, dtype, a.n, staged);
+    const bool tma = !int8 && !tile && aloco::use_tma(o.pass, M, dtype, staged);
     const bool fused = int8 && aloco::use_int8_fused(o.pass, M, dtype);
     if (fused || tile) {
         plan.grid = 0;

@@ -13,8 +13,9 @@ cudaError_t launch_int8_fused(const SyncArgs &a, const Int8Parts &P, aloco_dtype
                               int sm_count, int max_grid, cudaStream_t stream,
                               int *grid_out) {
     if (!int8_fused_fits(a.M, dtype)) return cudaErrorInvalidValue;
-    // A part that starts off a multiple of kPad puts all its blocks off 16-byte
-    // boundaries; the instances that stage such blocks as windows then run.
+    // A part that starts off a multiple of kPad (from the vector's first
+    // aligned element) puts all its blocks off 16-byte boundaries; the
+    // instances that stage such blocks as windows then run.
     bool odd = false;
     for (int p = 0; a.nvec > 0 && p < P.n_parts; ++p)
         odd = odd || (P.off[p] & (kPad - 1)) != 0;

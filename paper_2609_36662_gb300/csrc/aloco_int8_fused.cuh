@@ -706,7 +706,8 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
     // (the buffers are 16-byte aligned where a.nvec > 0)
     auto bulk_block = [&](int64_t s, int l) {
         if constexpr (ODD)
-            return l == kI8Block && a.nvec > 0 && (shift(s) == 0 || window(s) + kSlot <= a.n);
+            return l == kI8Block && a.nvec > 0 &&
+                   (shift(s) == 0 || (window(s) >= -a.head && window(s) + kSlot <= a.n));
         else
             return l == kI8Block && a.nvec > 0 && (s % kPad) == 0;
     };

@@ -41,9 +41,11 @@ struct SyncArgs {
     float *g;                       // theta [n]
     float *v;                       // momentum [n]
     void *x[ALOCO_MAX_WORKERS];     // replicas [n] each
-    int64_t n;                      // elements
-    int64_t nvec;                   // packs handled by the vector loop
-                                    // (0 when a buffer is not 16 B aligned)
+    int64_t n;                      // elements from the pointers on
+    int64_t nvec;                   // packs handled by the vector loop (0 when
+                                    // no element has all buffers 16 B aligned)
+    int head;                       // elements before the pointers (see
+                                    // set_buffers); 0 for aligned buffers
     // Round coefficients, each as an fp32 pair hi + lo whose sum carries the
     // fp64 host value to ~2^-48 relative, so that the per-element update is
     // not biased by one fixed fp32 rounding of the coefficient.
@@ -186,6 +188,13 @@ cudaError_t launch_adamw(const AdamArgs &a, aloco_dtype param_dtype,
                          aloco_dtype grad_dtype, int g2, cudaStream_t stream);
 
 // Host helpers shared by the entry points (aloco_host.cpp).
+// Fill a's buffers, n, nvec and head for the N elements that global,
+// momentum and locals point to.  Where every buffer reaches a 16-byte boundary
+// at the same element (views cut from aligned vectors at one ragged place),
+// the pointers start at that element and the head elements before it lie at
+// negative indices; the packs then serve all but the ends.
+void set_buffers(SyncArgs *a, float *global, float *momentum, void *const *locals,
+                 size_t N, int M, aloco_dtype dtype);
 int report_error(int code, const char *msg);
 // (base, index >= 0: the message names base[index])
 int check_buffer(const void *p, size_t bytes, int device, const char *base, int index = -1);

@@ -180,16 +180,7 @@ extern "C" int aloco_sync_noalloc(float *global, float *momentum,
 
     aloco::SyncArgs a;
     std::memset(&a, 0, sizeof a);
-    a.g = global;
-    a.v = momentum;
-    uintptr_t align_or = (uintptr_t)global | (uintptr_t)momentum;
-    for (int m = 0; m < M; ++m) {
-        a.x[m] = locals[m];
-        align_or |= (uintptr_t)locals[m];
-    }
-    const int pack = aloco::pack_elems(dtype);
-    a.n = (int64_t)N;
-    a.nvec = (align_or & 15) == 0 ? (int64_t)(N / pack) : 0;
+    aloco::set_buffers(&a, global, momentum, locals, N, M, dtype);
     aloco::split_coef(corr.inv_norm / (double)M, &a.c_hi, &a.c_lo);
     aloco::split_coef(corr.mu_t, &a.mu_hi, &a.mu_lo);
     aloco::split_coef(-corr.eta_out, &a.neg_eta_hi, &a.neg_eta_lo);
@@ -198,8 +189,9 @@ extern "C" int aloco_sync_noalloc(float *global, float *momentum,
     const int64_t work = a.nvec > 0 ? a.nvec : a.n;
     aloco::LaunchPlan plan;
     // the same choice of kernel as aloco_sync_ex
-    const bool tile = aloco::use_tile(o.pass, M, dtype, a.n, a.nvec);
-    const bool tma = !tile && aloco::use_tma(o.pass, M, dtype, a.nvec);
+    const int64_t staged = a.head == 0 ? a.nvec : 0;
+    const bool tile = aloco::use_tile(o.pass, M, dtype, a.n, staged);
+    const bool tma = !tile && aloco::use_tma(o.pass, M, dtype, staged);
     plan.grid = 0;
     plan.block = 0;
     plan.kernel = nullptr;

@@ -124,6 +124,37 @@ def test_unaligned_buffers(dt, offset):
     compare_round(wN, st, orc, g, v, xs)
 
 
+@pytest.mark.parametrize("int8", [False, True], ids=["plain", "int8"])
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+@pytest.mark.parametrize("offset", range(1, 9))
+@pytest.mark.parametrize("N", [3, 9, 4099, 1_300_007])
+def test_views_at_one_offset_equal_aligned_buffers(N, offset, dt, int8):
+    """Views cut at the same element of aligned vectors reach a 16-byte
+    boundary together, and the round runs packs behind a head of elements:
+    bit for bit the aligned round, nothing outside the views touched."""
+    w = W.small(N, 5, dt, seed=N % 89 + offset)
+    g, v, xs = gpu_inputs(w)
+    v.normal_(0, 1e-3, generator=torch.Generator("cuda").manual_seed(N))
+
+    def at(t):
+        whole = torch.full((offset + N + 9,), 3.5, dtype=t.dtype, device="cuda")
+        whole[offset:offset + N] = t
+        return whole, whole[offset:offset + N]
+    pairs = [at(t) for t in (g, v, *xs)]
+    kw = dict(H_sel=w.H_sel[0], H_base=w.H_base, step=w.start_step,
+              schedule=schedule_pair(w.schedule)[0], outer_lr=w.outer_lr,
+              outer_beta=w.outer_beta)
+    run = A.sync_int8 if int8 else A.sync
+    a = run(g, v, xs, **kw)
+    b = run(pairs[0][1], pairs[1][1], [p[1] for p in pairs[2:]], **kw)
+    assert a["status"] == b["status"] == A.OK
+    for want, (whole, got) in zip((g, v, *xs), pairs):
+        assert torch.equal(want, got)
+        assert bool((whole[:offset] == 3.5).all()) and bool((whole[offset + N:] == 3.5).all())
+    np.testing.assert_allclose(a["drift"], b["drift"], rtol=1e-6)
+    assert a["C"] == pytest.approx(b["C"], rel=1e-6)
+
+
 @pytest.mark.parametrize("pass_", [A.PASS_TILE, A.PASS_BULK_COPY], ids=["tile", "bulk_copy"])
 def test_bulk_passes_fall_back_on_unaligned_buffers(pass_):
     """The bulk-copy passes need 16-byte aligned buffers: asked for on a
