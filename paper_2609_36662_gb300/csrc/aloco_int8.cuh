@@ -279,6 +279,12 @@ __device__ __forceinline__ float2 mul2_rn(float2 a, float2 b) {
     return r;
 }
 
+// max(a, b, c), NaN if any operand is NaN
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
 // Half-integer margin of the product test below: 0.5 - 2^-14, exact in fp32.
 constexpr float kCodeMargin = 0.5f - 0x1p-14f;
 

@@ -450,12 +450,6 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-// max(a, b, c), NaN if any operand is NaN
-__device__ __forceinline__ float max3_nan(float a, float b, float c) {
-    float r;
-    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-    return r;
-}
 // Codes of a pair from the product y r (as code2_fast), with the distance
 // of each product from its nearest integer folded into `far`: the codes are
 // the codec's when far < kCodeMargin at the end (a NaN or infinite product

@@ -71,6 +71,35 @@ def test_codec_bit_exact(parts_name, kind):
     assert A.int8_num_blocks(parts or [N]) == O.int8_blocks(parts or [N])
 
 
+@pytest.mark.parametrize("shift", [0, 1, 4])
+@pytest.mark.parametrize("parts", [None, [3, 700 * 4096 + 5, 1, 769, 1100 * 4096, 4096 * 2 + 8]],
+                         ids=["one_part", "odd_parts"])
+def test_codec_runs_of_blocks(parts, shift):
+    """Vectors of more blocks than CTAs, so that CTAs walk runs of blocks
+    across part ends, from aligned and unaligned buffers: bit for bit the
+    oracle's."""
+    N = sum(parts) if parts else 1900 * 4096 + 77
+    y = _vec(N, 9)
+    whole = torch.zeros(N + shift, device="cuda")
+    whole[shift:] = torch.from_numpy(y)
+    codes, scales, dec = A.int8_encode(whole[shift:], parts)
+    oc, osc, odec = O.int8_encode(y, parts)
+    np.testing.assert_array_equal(codes.cpu().numpy(), oc)
+    _same_bits(scales.cpu().numpy(), osc)
+    _same_bits(dec.cpu().numpy(), odec)
+    bytes_ = torch.zeros(N + shift, dtype=torch.int8, device="cuda")
+    bytes_[shift:] = codes
+    _same_bits(A.int8_decode(bytes_[shift:], scales, parts).cpu().numpy(), odec)
+
+
+def test_decode_of_every_byte():
+    """Codes from a peer may hold any byte, -128 too, under any scale."""
+    codes = torch.arange(-128, 128, dtype=torch.int8, device="cuda").repeat(48)
+    scales = torch.tensor([0.37, float("inf"), float("nan")], device="cuda")
+    want = codes.float() * scales.repeat_interleave(4096)
+    _same_bits(A.int8_decode(codes, scales).cpu().numpy(), want.cpu().numpy())
+
+
 def _int8_oracle(w, g, v, xs, parts, step, hsel):
     corr = oracle_corr(w, step, hsel)
     dt = O.F32 if w.dtype == "f32" else O.BF16
