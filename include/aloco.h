@@ -120,7 +120,8 @@ typedef enum {
  *              aligned buffers, N >= 4096; otherwise REGISTERS runs);
  *   AUTO       the fastest as measured on GB300 for (M, dtype, N): TILE
  *              from 2^27 parameters for bf16 replicas with M <= 12 and for
- *              fp32 with M = 1 or 5..16, else REGISTERS.
+ *              fp32 with M = 1 or 5..16, and from 2^22 parameters for M > 16
+ *              (aligned buffers), else REGISTERS.
  * The INT8-communicated round (aloco_sync_int8) has two forms of its own:
  *   INT8_SPLIT a block-scale kernel, then an apply kernel that reads the
  *              replicas again (any M <= 16);

@@ -364,8 +364,14 @@ bool use_int8_fused(int pass, int M, aloco_dtype dtype) {
 
 bool use_tile(int pass, int M, aloco_dtype dtype, int64_t n, int64_t nvec) {
     if (!sync_tile_fits(M, n, nvec)) return false;
-    if (pass == ALOCO_PASS_TILE) return true;
+    if (pass == ALOCO_PASS_TILE) return M <= 16;
     if (pass != ALOCO_PASS_AUTO) return false;
+    // M = 17..32, against the register pass (one block per SM, whose loads in
+    // flight do not cover HBM latency): 6e6 x 32 bf16 0.77 against 0.73 of the
+    // copy peak, x 17 0.72 against 0.62, 6.4e7 x 32 bf16 0.96 against 0.85, fp32
+    // 0.99 against 0.84; at 2e6 they tie for bf16, and fp32 with 24 and 32
+    // workers is 4-7 % slower.
+    if (M > 16) return n >= (1 << 22);
     // AUTO, as measured on GB300 (fraction of the measured copy peak): from
     // 2^27 parameters the tile pass leads for bf16 replicas (0.97-0.98
     // against 0.94) and for fp32 with M = 1 or M >= 5 (0.96-0.98 against

@@ -1,5 +1,5 @@
 // Fused outer-synchronisation pass staged through shared memory by bulk
-// copies (the "tile" pass; M <= 16, 16-byte aligned buffers).
+// copies (the "tile" pass; 16-byte aligned buffers).
 //
 // The arithmetic per element is the register-streaming pass's (Algorithm 1:
 // Delta_m = theta - x_m summed in worker order; the drift energies and
@@ -35,7 +35,6 @@ namespace aloco {
 
 namespace {
 
-constexpr int kTileMaxM = 16;
 constexpr int kTileFlushBlocks = 8;
 constexpr size_t kTileSmemPerSm = 233472;   // shared memory of one SM
 constexpr size_t kTileSmemReserved = 1024;  // reserved by the system per CTA
@@ -128,24 +127,35 @@ __host__ __device__ constexpr bool tile_gv() {
 
 }  // namespace
 
-template <int M, bool BF16, int T, int NS>
-__global__ void __launch_bounds__(T, (tile_ctas<M, BF16, T>()))
+// M = 17..32 (MT = 0: the worker count comes with the arguments, and the
+// loops over workers are unrolled to 32 with uniform exits): 256-thread CTAs
+// with one stage of 1024 elements, as many per SM as their stages leave room
+// for (two for 32 bf16 workers, one for 32 fp32 workers), with the fp32
+// output tiles.  The register pass at these M holds one 256-thread block per
+// SM, whose loads in flight do not cover HBM latency: 6e6 x 32 bf16 166 us
+// against 151 here (the kernel).
+constexpr int kWideT = 256;
+
+template <int MT, bool BF16, int T, int NS>
+__global__ void __launch_bounds__(T, (MT == 0 ? 2 : tile_ctas<MT, BF16, T>()))
     sync_tile_kernel(const __grid_constant__ SyncArgs a) {
+    constexpr int MM = MT > 0 ? MT : ALOCO_MAX_WORKERS;
+    const int M = MT > 0 ? MT : a.M;
     constexpr int W = T / 32;
     constexpr int B = 4 * T;  // elements per block
     constexpr int ES = tile_es<BF16>();
-    constexpr bool GV = tile_gv<M, BF16, T, NS>();
+    constexpr bool GV = MT == 0 || tile_gv<MM, BF16, T, NS>();
     constexpr uint32_t kF = B * 4;   // one fp32 array of a block
     constexpr uint32_t kX = B * ES;  // one replica slice
-    constexpr uint32_t kStage = 2 * kF + M * kX;
+    const uint32_t kStage = 2 * kF + M * kX;
     constexpr uint32_t kOut = (uint32_t)tile_out_bytes<BF16, T, GV>();
 
-    __shared__ double e_w[W][M + 1];  // [warp][worker energies, then sum S^2]
+    __shared__ double e_w[W][MM + 1];  // [warp][worker energies, then sum S^2]
     __shared__ __align__(8) unsigned long long full_bar[NS];
     extern __shared__ __align__(128) unsigned char smem[];
 
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    if (lane < M) e_w[warp][lane] = 0.0;
+    if (lane < MM) e_w[warp][lane] = 0.0;
     if (t == 0) {
 #pragma unroll
         for (int s = 0; s < NS; ++s) mbar_init(smem_addr(&full_bar[s]), 1);
@@ -153,18 +163,26 @@ __global__ void __launch_bounds__(T, (tile_ctas<M, BF16, T>()))
     }
     __syncthreads();
 
-    float e_acc[M];
+    float e_acc[MM];
 #pragma unroll
-    for (int m = 0; m < M; ++m) e_acc[m] = 0.f;
+    for (int m = 0; m < MM; ++m) e_acc[m] = 0.f;
     int since_flush = 0;
     auto flush = [&]() {
+        if constexpr (MT == 0) {
+            // lane m gets worker m's warp sum
+            e_w[warp][lane] += (double)warp_sum_scatter<MM>(e_acc);
 #pragma unroll
-        for (int m = 0; m < M; ++m) {
-            float e = e_acc[m];
+            for (int m = 0; m < MM; ++m) e_acc[m] = 0.f;
+        } else {
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) e += __shfl_down_sync(0xffffffffu, e, off);
-            if (lane == 0) e_w[warp][m] += (double)e;
-            e_acc[m] = 0.f;
+            for (int m = 0; m < MM; ++m) {
+                float e = e_acc[m];
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1)
+                    e += __shfl_down_sync(0xffffffffu, e, off);
+                if (lane == 0) e_w[warp][m] += (double)e;
+                e_acc[m] = 0.f;
+            }
         }
         since_flush = 0;
     };
@@ -192,9 +210,10 @@ __global__ void __launch_bounds__(T, (tile_ctas<M, BF16, T>()))
         bulk_load(smem_addr(st), a.g + kb * B, kF, bar);
         bulk_load(smem_addr(st + kF), a.v + kb * B, kF, bar);
 #pragma unroll
-        for (int m = 0; m < M; ++m)
-            bulk_load(smem_addr(st + 2 * kF + m * kX),
-                      reinterpret_cast<const unsigned char *>(a.x[m]) + kb * B * ES, kX, bar);
+        for (int m = 0; m < MM; ++m)
+            if (MT > 0 || m < M)
+                bulk_load(smem_addr(st + 2 * kF + m * kX),
+                          reinterpret_cast<const unsigned char *>(a.x[m]) + kb * B * ES, kX, bar);
     };
     // thread 0: block j's output tiles to global memory
     auto store_tiles = [&](int64_t j) {
@@ -206,9 +225,10 @@ __global__ void __launch_bounds__(T, (tile_ctas<M, BF16, T>()))
             bulk_store(a.v + kb * B, smem_addr(og + kF), kF);
         }
 #pragma unroll
-        for (int m = 0; m < M; ++m)
-            bulk_store(reinterpret_cast<unsigned char *>(a.x[m]) + kb * B * ES, smem_addr(ob),
-                       kX);
+        for (int m = 0; m < MM; ++m)
+            if (MT > 0 || m < M)
+                bulk_store(reinterpret_cast<unsigned char *>(a.x[m]) + kb * B * ES, smem_addr(ob),
+                           kX);
         bulk_commit();
     };
 
@@ -231,7 +251,8 @@ __global__ void __launch_bounds__(T, (tile_ctas<M, BF16, T>()))
         const float vv[4] = {v4.x, v4.y, v4.z, v4.w};
         float sm[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int m = 0; m < M; ++m) {
+        for (int m = 0; m < MM; ++m) {
+            if (MT == 0 && m >= M) break;
             float xx[4];
             const unsigned char *xp = st + 2 * kF + m * kX + 4 * t * ES;
             if constexpr (BF16) {
@@ -319,7 +340,8 @@ __global__ void __launch_bounds__(T, (tile_ctas<M, BF16, T>()))
             const float v = a.v[jj];
             float s = 0.f;
 #pragma unroll
-            for (int m = 0; m < M; ++m) {
+            for (int m = 0; m < MM; ++m) {
+                if (MT == 0 && m >= M) break;
                 float x;
                 if constexpr (BF16)
                     x = __uint_as_float(
@@ -337,7 +359,8 @@ __global__ void __launch_bounds__(T, (tile_ctas<M, BF16, T>()))
             a.g[jj] = gp;
             a.v[jj] = vp;
 #pragma unroll
-            for (int m = 0; m < M; ++m) {
+            for (int m = 0; m < MM; ++m) {
+                if (MT == 0 && m >= M) break;
                 if constexpr (BF16)
                     reinterpret_cast<__nv_bfloat16 *>(a.x[m])[jj] = __float2bfloat16_rn(gp);
                 else
@@ -350,8 +373,8 @@ __global__ void __launch_bounds__(T, (tile_ctas<M, BF16, T>()))
     b64 += (double)b32;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) b64 += __shfl_down_sync(0xffffffffu, b64, off);
-    if (lane == 0) e_w[warp][M] = b64;
-    finish_rows<M, W>(a, M, e_w, nf);
+    if (lane == 0) e_w[warp][MM] = b64;
+    finish_rows<MM, W>(a, M, e_w, nf);
 }
 
 namespace {
@@ -388,6 +411,40 @@ cudaError_t tile_launch(const SyncArgs &a, int sm_count, int max_grid, cudaStrea
     return cudaGetLastError();
 }
 
+// M = 17..32
+template <bool BF16>
+cudaError_t wide_launch(const SyncArgs &a, int sm_count, int max_grid, cudaStream_t stream,
+                        int *grid_out) {
+    const auto kernel = sync_tile_kernel<0, BF16, kWideT, 1>;
+    const size_t stage = (size_t)4 * kWideT * (8 + a.M * tile_es<BF16>());
+    const size_t smem = stage + 2 * tile_out_bytes<BF16, kWideT, true>();
+    constexpr size_t kMost = (size_t)4 * kWideT * (8 + ALOCO_MAX_WORKERS * tile_es<BF16>()) +
+                             2 * tile_out_bytes<BF16, kWideT, true>();
+    static_assert(kMost + (kWideT / 32) * (ALOCO_MAX_WORKERS + 2) * 8 + 256 <=
+                      kTileSmemPerSm - kTileSmemReserved,
+                  "the stage of 32 workers exceeds shared memory");
+    static PerDevice occ_cache[ALOCO_MAX_WORKERS + 1];  // by worker count
+    const int dev = PerDevice::device();
+    int occ = occ_cache[a.M].get(dev);
+    if (occ == 0) {
+        cudaError_t e = cudaFuncSetAttribute(
+            kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kWideT, smem);
+        if (e != cudaSuccess) return e;
+        if (occ < 1) occ = 1;
+        occ_cache[a.M].set(dev, occ);
+    }
+    const int64_t nblk = a.n / (4 * kWideT);
+    int64_t grid = (int64_t)sm_count * occ;
+    if (grid > nblk) grid = nblk;
+    if (grid > max_grid) grid = max_grid;
+    if (grid < 1) grid = 1;
+    *grid_out = (int)grid;
+    kernel<<<(unsigned)grid, kWideT, smem, stream>>>(a);
+    return cudaGetLastError();
+}
+
 template <bool BF16>
 cudaError_t tile_dispatch(const SyncArgs &a, int sm_count, int max_grid, cudaStream_t stream,
                           int *grid_out) {
@@ -407,7 +464,8 @@ cudaError_t tile_dispatch(const SyncArgs &a, int sm_count, int max_grid, cudaStr
         case 13: return tile_launch<13, BF16>(a, sm_count, max_grid, stream, grid_out);
         case 14: return tile_launch<14, BF16>(a, sm_count, max_grid, stream, grid_out);
         case 15: return tile_launch<15, BF16>(a, sm_count, max_grid, stream, grid_out);
-        default: return tile_launch<16, BF16>(a, sm_count, max_grid, stream, grid_out);
+        case 16: return tile_launch<16, BF16>(a, sm_count, max_grid, stream, grid_out);
+        default: return wide_launch<BF16>(a, sm_count, max_grid, stream, grid_out);
     }
 }
 
@@ -415,7 +473,7 @@ cudaError_t tile_dispatch(const SyncArgs &a, int sm_count, int max_grid, cudaStr
 
 bool sync_tile_fits(int M, int64_t n, int64_t nvec) {
     // at least one whole block of the largest shape (4 x 1024 elements)
-    return M >= 1 && M <= kTileMaxM && nvec > 0 && n >= 4096;
+    return M >= 1 && M <= ALOCO_MAX_WORKERS && nvec > 0 && n >= 4096;
 }
 
 cudaError_t launch_sync_tile(const SyncArgs &a, aloco_dtype dtype, int sm_count, int max_grid,

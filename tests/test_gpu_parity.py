@@ -378,6 +378,29 @@ def test_tile_pass_equals_register_pass_bit_for_bit(M, dt):
         assert s1["drift"][m] == pytest.approx(s2["drift"][m], rel=RTOL_STAT)
 
 
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+@pytest.mark.parametrize("M", [17, 24, 32])
+@pytest.mark.parametrize("N", [1 << 22, (1 << 22) + 1023, 6_000_001])
+def test_wide_tile_pass_equals_register_pass_bit_for_bit(N, M, dt):
+    """AUTO's tile pass above 16 workers, at its smallest size, with ragged
+    ends and with several blocks to a CTA."""
+    w = W.small(N, M, dt, seed=M)
+    outs = []
+    for p in (A.PASS_REGISTERS, A.PASS_AUTO):
+        g, v, xs = gpu_inputs(w)
+        v.normal_(0, 1e-3, generator=torch.Generator("cuda").manual_seed(M))
+        st = run_gpu_round(g, v, xs, w, w.start_step, w.H_sel[0],
+                           opts=A.default_opts(pass_=p))
+        assert st["status"] == A.OK
+        outs.append((st, g, v, xs))
+    (s1, g1, v1, x1), (s2, g2, v2, x2) = outs
+    assert (s1["pass_used"], s2["pass_used"]) == (A.PASS_REGISTERS, A.PASS_TILE)
+    assert torch.equal(g1, g2) and torch.equal(v1, v2)
+    assert all(torch.equal(a, b) for a, b in zip(x1, x2))
+    np.testing.assert_allclose(s1["drift"], s2["drift"], rtol=RTOL_STAT)
+    assert s1["mean_sq_norm"] == pytest.approx(s2["mean_sq_norm"], rel=RTOL_STAT)
+
+
 def test_auto_pass_choice():
     """AUTO runs the tile pass from 2^27 parameters for fp32 with M = 1 or
     5..16 and for bf16 with M <= 12, and the register pass elsewhere (fp32
