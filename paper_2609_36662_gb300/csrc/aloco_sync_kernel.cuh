@@ -173,6 +173,31 @@ struct Pack<true> {
     }
 };
 
+// A sum as an unevaluated pair of floats, hi + lo: adding two keeps the
+// rounding error of hi exactly (the two-sum of Knuth, TAOCP 4.2.2) and leaves
+// about 2^-46 of the sum in lo.  Ten fp32 additions, a small part of what
+// one fp64 addition costs here.  hi must not overflow.
+struct FloatPair {
+    float hi, lo;
+};
+__device__ __forceinline__ FloatPair operator+(FloatPair a, FloatPair b) {
+    const float s = __fadd_rn(a.hi, b.hi);
+    const float t = __fsub_rn(s, a.hi);
+    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, t)), __fsub_rn(b.hi, t));
+    return {s, __fadd_rn(__fadd_rn(a.lo, b.lo), e)};
+}
+__device__ __forceinline__ double value(FloatPair a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double value(double a) { return a; }
+__device__ __forceinline__ float from_lane_xor(float v, int mask) {
+    return __shfl_xor_sync(0xffffffffu, v, mask);
+}
+__device__ __forceinline__ double from_lane_xor(double v, int mask) {
+    return __shfl_xor_sync(0xffffffffu, v, mask);
+}
+__device__ __forceinline__ FloatPair from_lane_xor(FloatPair v, int mask) {
+    return {__shfl_xor_sync(0xffffffffu, v.hi, mask), __shfl_xor_sync(0xffffffffu, v.lo, mask)};
+}
+
 // Warp sums of the P values each lane holds (P a power of two, at most 32)
 // by recursive halving: at each step a lane keeps the half of its values
 // that its lane bit selects and adds the partner's copy of that half; the
@@ -193,10 +218,10 @@ __device__ __forceinline__ T warp_sum_scatter(T (&v)[P]) {
             for (int i = 0; i < n / 2; ++i) {
                 const T send = up ? v[i] : v[i + n / 2];
                 const T keep = up ? v[i + n / 2] : v[i];
-                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
+                v[i] = keep + from_lane_xor(send, mask);
             }
         } else {
-            v[0] += __shfl_xor_sync(0xffffffffu, v[0], mask);
+            v[0] = v[0] + from_lane_xor(v[0], mask);
         }
     }
     return v[0];
@@ -244,9 +269,14 @@ __device__ __forceinline__ void finish_rows(const SyncArgs &a, int M, double (&r
     const unsigned long long nfl = warp_sum(nf);
     if (lane == 0) shnf[warp] = nfl;
     __syncthreads();
-    for (int p = warp; p < np; p += NW) {
-        const double v = column_sum(rows, NW, slot(p));
-        if (lane == 0) a.partials[(int64_t)blockIdx.x * np + p] = v;
+    // the NW rows of 32 / R columns in one warp at a time
+    constexpr int R = pow2_at_least(NW), C = 32 / R;
+    for (int p0 = warp * C; p0 < np; p0 += NW * C) {
+        const int p = p0 + lane / R, w = lane % R;
+        double v = w < NW && p < np ? rows[w][slot(p)] : 0.0;
+#pragma unroll
+        for (int off = R / 2; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (w == 0 && p < np) a.partials[(int64_t)blockIdx.x * np + p] = v;
     }
     if (t == kThreads - 1) {
         unsigned long long n = 0;
@@ -324,22 +354,26 @@ __device__ __forceinline__ void finish_rows(const SyncArgs &a, int M, double (&r
 // thread and a serial publish: 2^20 parameters x 4 fp32 workers 20.0 -> 15.1
 // us (the kernel, ncu), 6e6 x 32 bf16 190 -> 166 us; the fused INT8 kernel, 1024
 // threads a block, 2e7 x 16 bf16 385 -> 300 us, 2e7 x 8 fp32 330 -> 283 us.  S bounds the rows where shared memory is short.
+template <int MM, typename T>
+__device__ __forceinline__ void fold_warp(double (&row)[MM + 1], const T (&e)[MM], T b) {
+    constexpr int P = pow2_at_least(MM);
+    const int lane = threadIdx.x & 31;
+    T v[P];
+#pragma unroll
+    for (int m = 0; m < P; ++m) v[m] = m < MM ? e[m < MM ? m : 0] : T{};
+    const double sum = value(warp_sum_scatter<P>(v));
+    const int w = lane / (32 / P);
+    if (lane % (32 / P) == 0 && w < MM) row[w] = sum;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) b = b + from_lane_xor(b, off);
+    if (lane == 0) row[MM] = value(b);
+}
 template <int MM, int NW, int S = 32>
 __device__ __forceinline__ void reduce_and_finish(const SyncArgs &a, int M,
                                                   double (&e64)[MM], double b64,
                                                   unsigned nf) {
-    constexpr int P = pow2_at_least(MM);
     __shared__ double rows[S][MM + 1];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double v[P];
-#pragma unroll
-    for (int m = 0; m < P; ++m) v[m] = m < MM ? e64[m < MM ? m : 0] : 0.0;
-    const double e = warp_sum_scatter<P>(v);
-    const int w = lane / (32 / P);
-    if (lane % (32 / P) == 0 && w < MM) rows[warp][w] = e;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) b64 += __shfl_down_sync(0xffffffffu, b64, off);
-    if (lane == 0) rows[warp][MM] = b64;
+    fold_warp<MM>(rows[threadIdx.x >> 5], e64, b64);
     finish_rows<MM, NW>(a, M, rows, nf);
 }
 
@@ -521,9 +555,28 @@ __global__ void __launch_bounds__(kBlock, (min_blocks<MT, BF16>()))
             cnt = 0;
         }
     }
-    flush();
-
-    reduce_and_finish<MM, kBlock / 32>(a, M, e64, b64, nf);
+    // A small round: no thread has come to a flush, so its sums are the fp32
+    // partials, and a warp adds them as float pairs instead of doubles (which
+    // took 3 to 5 us of a round: the flush and the warp's sums, with the fp64
+    // pipe of an SM at two additions a clock; the kernel at 2^20 parameters: 8 fp32
+    // workers 22.5 -> 18.1 us, 4 16.8 -> 14.5, 16 bf16 25.0 -> 22.9).  Partials above 2^100, whose
+    // pair could overflow, infinities and NaN take the doubles.
+    const int64_t loose = a.head + a.n - a.nvec * PACK;
+    const bool small = (a.nvec + stride - 1) / stride + (loose + stride - 1) / stride < kFlush;
+    float top = b32;
+#pragma unroll
+    for (int m = 0; m < MM; ++m) top = e32[m] <= 0x1p100f ? top : e32[m];
+    __shared__ double rows[32][MM + 1];
+    if (small && __all_sync(0xffffffffu, top <= 0x1p100f)) {
+        FloatPair pairs[MM];
+#pragma unroll
+        for (int m = 0; m < MM; ++m) pairs[m] = {e32[m], 0.f};
+        fold_warp<MM>(rows[threadIdx.x >> 5], pairs, FloatPair{b32, 0.f});
+    } else {
+        flush();
+        fold_warp<MM>(rows[threadIdx.x >> 5], e64, b64);
+    }
+    finish_rows<MM, kBlock / 32>(a, M, rows, nf);
 }
 
 // Tuned residency (blocks of kBlock threads per SM) of the fused pass for

@@ -401,6 +401,24 @@ def test_wide_tile_pass_equals_register_pass_bit_for_bit(N, M, dt):
     assert s1["mean_sq_norm"] == pytest.approx(s2["mean_sq_norm"], rel=RTOL_STAT)
 
 
+@pytest.mark.parametrize("size", [1e-17, 1.0, 5e18])
+@pytest.mark.parametrize("N", [1000, 1_500_001, 11_000_000])
+def test_energies_over_the_whole_float_range(N, size):
+    """Energies of tiny and huge pseudo-gradients: a thread's fp32 partial is
+    finite, the sums over a warp and a block need not fit a float (small
+    rounds add float pairs, with doubles beyond 2^100)."""
+    w = W.small(N, 1, "f32", seed=5)
+    gen = torch.Generator("cuda").manual_seed(N)
+    g = torch.zeros(N, device="cuda").normal_(0, size, generator=gen).clamp_(-size, size)
+    x = torch.zeros(N, device="cuda")
+    v = torch.zeros(N, device="cuda")
+    energy = float(g.double().square().sum())
+    st = run_gpu_round(g, v, [x], w, w.start_step, w.H_sel[0])
+    assert st["status"] == A.OK
+    assert st["D"] == pytest.approx(energy, rel=RTOL_STAT)
+    assert st["mean_sq_norm"] == pytest.approx(energy, rel=RTOL_STAT)
+
+
 def test_auto_pass_choice():
     """AUTO runs the tile pass from 2^27 parameters for fp32 with M = 1 or
     5..16 and for bf16 with M <= 12, and the register pass elsewhere (fp32
