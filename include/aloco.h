@@ -279,11 +279,13 @@ int aloco_sync_ex(float *global, float *momentum, void *const *locals,
 /* One outer round (as aloco_sync_ex, Algorithm 1) on state that lives in
  * host memory: theta, v and the M replicas are page-locked host arrays
  * (cudaMallocHost, or registered with cudaHostRegister); any other memory
- * is ALOCO_ERR_ARG.  The library streams them through cached device
- * staging in chunks of chunk_elems elements (0 = 2^24; rounded up to a
- * multiple of 8), overlapping the host-to-device copy of one chunk, the
- * fused kernel on another and the device-to-host copy of theta' and v' of a
- * third, on two internal copy streams and opts->stream.
+ * is ALOCO_ERR_ARG.  With chunk_elems = 0 and buffers that reach a 16-byte
+ * boundary at the same element, one kernel reads and writes them over the
+ * host link, without staging.  Otherwise the library streams them through
+ * cached device staging in chunks of chunk_elems elements (0 = 2^24; rounded
+ * up to a multiple of 8), overlapping the host-to-device copy of one chunk,
+ * the fused kernel on another and the device-to-host copy of theta' and v' of
+ * a third, on two internal copy streams and opts->stream.
  *   global, momentum  in: theta, v; out: theta', v' (fp32, N each);
  *   locals            in only: the replicas' endpoints.  The host replicas
  *                     are NOT reset; the reset replicas equal theta', which
@@ -294,7 +296,7 @@ int aloco_sync_ex(float *global, float *momentum, void *const *locals,
  * pass runs (opts->pass AUTO or REGISTERS; BULK_COPY is ALOCO_ERR_ARG).
  * The call returns when theta', v' and the statistics are in place.  The
  * device staging (3 chunks of (8 + M * element size) bytes each) is
- * allocated on first use, kept until aloco_shutdown, and shared by the
+ * allocated on first use of chunks, kept until aloco_shutdown, and shared by the
  * device's calls, which therefore must not overlap. */
 int aloco_sync_host(float *global, float *momentum, const void *const *locals,
                     size_t N, int M, aloco_dtype dtype, int64_t H_sel,

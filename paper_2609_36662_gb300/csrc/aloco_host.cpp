@@ -995,6 +995,68 @@ int aloco_int8_decode(const int8_t *codes, const float *scales, size_t N,
     return ALOCO_OK;
 }
 
+// The host-memory round without staging: the register pass on the buffers'
+// device addresses, the replicas read only.  The host link bounds it, and the
+// loads and stores of one kernel keep both directions of the link busy from
+// the first pack to the last, where staged chunks copy in before anything
+// computes and out after it.  One block per SM: more gain nothing, and with
+// bf16 replicas, whose threads write theta' and v' as two 16-byte halves of
+// 32 bytes, the halves then reach the link apart (161 against 268 GB/s).  Calls,
+// staged (chunks of 2^24) against direct: 1e6 x 4 fp32 227 and 152 us, 5e6 x 4
+// fp32 889 and 622 us, 2e7 x 8 fp32 4461 and 3889 us, the 150M set x 4 bf16 13.0
+// and 12.1 ms (254 and 274 GB/s), x 8 fp32 28.8 and 26.5 ms.
+static int host_direct(Workspace *ws, aloco::SyncArgs &a, const aloco_correction_t &corr,
+                       aloco_dtype dtype, const aloco_opts_t &o, aloco_stats_t *st) {
+    const int M = st->M;
+    split_coef(corr.inv_norm / (double)M, &a.c_hi, &a.c_lo);
+    split_coef(corr.mu_t, &a.mu_hi, &a.mu_lo);
+    split_coef(-corr.eta_out, &a.neg_eta_hi, &a.neg_eta_lo);
+    a.M = M;
+    a.keep_x = 1;
+    a.partials = ws->partials;
+    a.nf_partials = ws->nf_partials;
+    a.ticket = ws->ticket;
+    a.totals = ws->totals;
+    a.nf_total = ws->nf_total;
+    a.error = ws->error;
+    a.stats_out = ws->stats_dev;
+    a.seq = ++ws->seq;
+    aloco::LaunchPlan plan;
+    const int bps = o.blocks_per_sm > 0 ? o.blocks_per_sm : 1;
+    cudaError_t e = dtype == ALOCO_F32
+                        ? aloco::plan_sync_f32(M, a.nvec, ws->sm_count, bps, &plan)
+                        : aloco::plan_sync_bf16(M, a.nvec, ws->sm_count, bps, &plan);
+    if (e != cudaSuccess) return cuda_fail(e, "launch plan");
+    cudaStream_t stream = (cudaStream_t)o.stream;
+    if (o.time_kernel) e = cudaEventRecord(ws->ev0, stream);
+    void *params[] = {&a};
+    if (e == cudaSuccess)
+        e = cudaLaunchKernel(plan.kernel, dim3(plan.grid), dim3(plan.block), params, plan.smem,
+                             stream);
+    if (e == cudaSuccess && o.time_kernel) e = cudaEventRecord(ws->ev1, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+    if (e != cudaSuccess) return cuda_fail(e, "host round");
+    const int rc = wait_published(ws->stats_host, a.seq, stream);
+    if (rc != ALOCO_OK) return rc;
+    unsigned long long nf;
+    std::memcpy(&nf, ws->stats_host + aloco::kNfSlot, sizeof nf);
+    finalize_stats(ws->stats_host, nf, M, o.eps, 1.0 / ((double)M * (double)M), st);
+    st->grid = plan.grid;
+    st->pass_used = ALOCO_PASS_REGISTERS;
+    if (o.time_kernel) {
+        float ms = -1.f;
+        if (cudaEventElapsedTime(&ms, ws->ev0, ws->ev1) == cudaSuccess)
+            st->kernel_ms = ms;
+        else
+            cudaGetLastError();
+    }
+    if (st->nonfinite > 0 || !std::isfinite(st->D) || !std::isfinite(st->C))
+        return fail(ALOCO_ERR_NONFINITE, "round produced %lld non-finite elements (D=%g, C=%g)",
+                    (long long)st->nonfinite, st->D, st->C);
+    t_err.clear();
+    return ALOCO_OK;
+}
+
 int aloco_sync_host(float *global, float *momentum, const void *const *locals,
                     size_t N, int M, aloco_dtype dtype, int64_t H_sel,
                     int64_t H_base, int64_t step, const aloco_schedule_t *schedule,
@@ -1045,9 +1107,12 @@ int aloco_sync_host(float *global, float *momentum, const void *const *locals,
     for (int m = 0; m < M; ++m)
         if ((uintptr_t)locals[m] & (rsz - 1))
             return fail(ALOCO_ERR_ARG, "locals[%d] not %zu-byte aligned", m, rsz);
+    bool mapped = false;  // every buffer has a device address
+    void *dev_ptrs[2 + ALOCO_MAX_WORKERS];
     {
         const void *ptrs[2 + ALOCO_MAX_WORKERS] = {global, momentum};
         for (int m = 0; m < M; ++m) ptrs[2 + m] = locals[m];
+        mapped = true;
         for (int i = 0; i < M + 2; ++i) {
             cudaPointerAttributes at;
             cudaError_t e = cudaPointerGetAttributes(&at, ptrs[i]);
@@ -1056,6 +1121,8 @@ int aloco_sync_host(float *global, float *momentum, const void *const *locals,
                 return fail(ALOCO_ERR_ARG,
                             "buffer %d is not page-locked host memory (allocate it with "
                             "cudaMallocHost or register it with cudaHostRegister)", i);
+            dev_ptrs[i] = at.devicePointer;
+            mapped = mapped && at.devicePointer;
         }
     }
     size_t chunk = chunk_elems ? chunk_elems : ((size_t)1 << 24);
@@ -1070,6 +1137,15 @@ int aloco_sync_host(float *global, float *momentum, const void *const *locals,
     std::lock_guard<std::mutex> lk(ws->mu);
     rc = ensure_ready(ws, device);
     if (rc != ALOCO_OK) return rc;
+
+    if (chunk_elems == 0 && mapped) {
+        // no staging: see host_direct
+        aloco::SyncArgs a;
+        std::memset(&a, 0, sizeof a);
+        aloco::set_buffers(&a, (float *)dev_ptrs[0], (float *)dev_ptrs[1], dev_ptrs + 2, N, M,
+                           dtype);
+        if (a.nvec > 0) return host_direct(ws, a, corr, dtype, o, st);
+    }
 
     // streams, events and staging (grown on demand, kept until shutdown)
     if (!ws->hs_in) {

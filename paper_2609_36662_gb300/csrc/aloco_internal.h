@@ -53,6 +53,7 @@ struct SyncArgs {
     float mu_hi, mu_lo;             // mu_t
     float neg_eta_hi, neg_eta_lo;   // -eta_out
     int M;
+    int keep_x;                     // 1: the replicas are read only (register pass)
     // workspace (device)
     double *partials;               // [grid][M + 1]: sum Delta_m^2 (m < M), sum S^2
     unsigned long long *nf_partials;// [grid]

@@ -445,11 +445,13 @@ __global__ void __launch_bounds__(kBlock, (min_blocks<MT, BF16>()))
         }
         P::store(a.g, i, gp);
         P::store(a.v, i, vp);
-        const typename P::Raw xo = P::narrow(gp);
+        if (!a.keep_x) {
+            const typename P::Raw xo = P::narrow(gp);
 #pragma unroll
-        for (int m = 0; m < MM; ++m) {
-            if (MT == 0 && m >= M) continue;
-            P::store_x(a.x[m], i, xo);
+            for (int m = 0; m < MM; ++m) {
+                if (MT == 0 && m >= M) continue;
+                P::store_x(a.x[m], i, xo);
+            }
         }
         if (++cnt == kFlush) {
             flush();
@@ -543,7 +545,7 @@ __global__ void __launch_bounds__(kBlock, (min_blocks<MT, BF16>()))
         a.v[j] = vp;
 #pragma unroll
         for (int m = 0; m < MM; ++m) {
-            if (MT == 0 && m >= M) continue;
+            if ((MT == 0 && m >= M) || a.keep_x) continue;
             if constexpr (BF16)
                 reinterpret_cast<__nv_bfloat16 *>(a.x[m])[j] =
                     __float2bfloat16_rn(gp);

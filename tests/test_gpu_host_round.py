@@ -114,3 +114,37 @@ def test_pageable_memory_and_bulk_copy_are_rejected():
         A.sync_host(_pinned(g), _pinned(v), [_pinned(x) for x in xs],
                     opts=A.default_opts(pass_=A.PASS_BULK_COPY), **kw)
     assert ei.value.status == A.ERR_ARG
+
+
+@pytest.mark.parametrize("chunk", [0, 4096])
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+@pytest.mark.parametrize("off,off_v", [(0, 0), (3, 3), (5, 5), (3, 2)])
+def test_host_round_on_views(off, off_v, dt, chunk):
+    """Views of page-locked vectors: cut at one element (read and written in
+    place, behind a head of elements) or at two (staged), the round equals the
+    device round bit for bit and touches nothing outside the views."""
+    N, M = 70_003, 3
+    w = W.small(N, M, dt, seed=9)
+    g, v, xs = gpu_inputs(w)
+    v.normal_(0, 1e-3, generator=torch.Generator("cuda").manual_seed(2))
+
+    def view(t, k):
+        whole = torch.full((N + 16,), 3.5, dtype=t.dtype).pin_memory()
+        whole[k:k + N] = t.cpu()
+        return whole, whole[k:k + N]
+    pairs = [view(g, off), view(v, off_v)] + [view(x, off) for x in xs]
+    x_before = [p[0].clone() for p in pairs[2:]]
+    sa, _ = schedule_pair(w.schedule)
+    kw = dict(H_sel=w.H_sel[0], H_base=w.H_base, step=w.start_step, schedule=sa,
+              outer_lr=w.outer_lr, outer_beta=w.outer_beta)
+    st_d = A.sync(g, v, xs, **kw)
+    st_h = A.sync_host(pairs[0][1], pairs[1][1], [p[1] for p in pairs[2:]],
+                       chunk_elems=chunk, **kw)
+    assert st_d["status"] == st_h["status"] == A.OK
+    for (whole, part), want, k in zip(pairs[:2], (g, v), (off, off_v)):
+        assert torch.equal(_bits(part), _bits(want.cpu()))
+        assert bool((whole[:k] == 3.5).all()) and bool((whole[k + N:] == 3.5).all())
+    for (whole, _), before in zip(pairs[2:], x_before):
+        assert torch.equal(_bits(whole), _bits(before))
+    assert st_h["D"] == pytest.approx(st_d["D"], rel=RTOL_STAT)
+    assert st_h["C"] == pytest.approx(st_d["C"], rel=RTOL_STAT)
