@@ -15,10 +15,10 @@
 //   1. theta, v and the M replica slices arrive in shared memory by bulk
 //      copies (cp.async.bulk, one per array, issued by thread 0 and
 //      completing on the CTA's mbarrier; every thread's wait on it is
-//      bounded).  Blocks off a 16-byte boundary come with a few elements
-//      before and after them (see kPad).  Short blocks (tensor ends) are
-//      instead staged by every thread, element by element, into its own
-//      slots;
+//      bounded).  In the ODD instances, blocks off a 16-byte boundary and
+//      short ones come as their windows (see kPad).  What no bulk copy serves
+//      (short blocks elsewhere, the vector's ends) is instead staged by every
+//      thread, element by element, into its own slots;
 //   2. each warp reduces every worker's max |Delta_m| (as float bits, NaN
 //      above +inf); barrier 1; every warp then reads the 32 warp maxima of
 //      each worker lane-parallel and folds them with one warp max, and lane
@@ -123,16 +123,21 @@ __host__ __device__ constexpr int esize() { return BF16 ? 2 : 4; }
 // aligned one.  The block's elements are window elements [sh, sh + 4096), sh
 // = start mod kPad; threads own slots 0..4095, and slot e stands for window
 // element e, or for element 4096 + e where e < sh.  Only slots 0..kPad - 1
-// (the first chunks of threads 0 and 1) hold elements at the window's ends:
-// those two threads move the wrapped elements into their slots when the
-// block lands and store their results themselves, and bulk copies store
-// window elements [kPad, 4096).  Bound by HBM like an aligned block; staged
-// element by element instead (what every such block took before, and blocks
-// at the vector's ends or shorter than 4096 still take) 20e6 parameters x 16
-// bf16 workers in parts of odd sizes ran at 0.22 of the copy peak.
+// (the first chunks of two threads) hold elements at the window's ends: those
+// threads move the wrapped elements into their slots when the block lands,
+// bulk copies store window elements [kPad, 4096) of the output tiles, and
+// the warps store the ends from the tiles.  A short block's window ends sooner, its
+// slots beyond are zeroed, and bulk copies store the whole packs.  Bound by
+// HBM like an aligned block.  Rounds of 2e7 parameters x 16 bf16 workers in 45
+// parts of odd sizes (whole calls): 1067 us element by element, 365 us with
+// windows for whole blocks and their ends stored by the two threads that
+// hold them, 352 us with windows for short blocks too and the ends stored by
+// the warps.  Against the same vector in one part (4e7 parameters, kernel):
+// 575 and 530 us at 16 bf16 workers, 539 and 436 at 12, 360 and 310 at 8; the
+// wrapped elements' moves cost 2-6 % of that, the ends up to 4 %.
 // The code for windows costs registers that some shapes do not have to spare
-// (bf16 M = 12: 182 bytes of spills against 88), so it is compiled only into
-// the ODD instances, which run when some part starts off a multiple of kPad.
+// and time some code (above), so it is compiled only into the ODD instances,
+// which run when some part starts off a multiple of kPad.
 constexpr int kPad = 8;
 constexpr int kSlot = kI8Block + kPad;  // elements of a staged array
 // Workers whose replica slices are staged at a time (a group), at most
@@ -591,14 +596,14 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
     constexpr uint32_t kGVBytes = kI8Block * 4;  // one fp32 array of a block
     constexpr uint32_t kXBytes = kI8Block * ES;  // one replica slice
     constexpr uint32_t kXSlot = kSlot * ES;      // its place in shared memory
-    constexpr uint32_t kPadGV = kPad * 4, kPadX = kPad * ES;  // a window's extra bytes
     // Single buffers suffice: red_w is read between a group's first barrier
     // and the next barrier, and rewritten only after it; red1 is read after
     // barrier 2 and rewritten only after the next block's first barrier.
     __shared__ unsigned red_w[G][W];                  // [worker][warp]: conflict-free reads
     __shared__ unsigned red1[W];
     __shared__ double e_w[W][M + 1];   // [warp][worker energies, then sum Dbar^2]
-    __shared__ int64_t s_pstart;        // thread 0: start of the block whose tiles wait
+    __shared__ int64_t s_pstart;        // thread 0: start and length of the block
+    __shared__ int s_plen;              // whose tiles wait
     // the next block's start and length, located by thread 0 as a block
     // starts and read by every thread after barrier 1 (two slots by the
     // parity of the iteration: a slot is rewritten only after every thread
@@ -668,12 +673,26 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
     const int nblocks = (int)P.blk[P.n_parts];  // below 2^31 - grid (host check)
     // thread t holds the 4-element chunks at 4t + c x 4T (c < PER / 4), so
     // every warp access to a staged array is contiguous
-    auto el = [&](int i) { return (i >> 2) * (4 * T) + 4 * t + (i & 3); };
-    // a block's offset in its window, the window's first element, and the
-    // window element that slot e stands for (see kPad)
+    // (in the ODD instances slot t belongs to thread t + 32: warp 1, not warp
+    // 0 with the copies' issue, holds the first chunks, which cost more)
+    const int ts = ODD ? (t + T - 32) % T : t;
+    auto el = [&](int i) { return (i >> 2) * (4 * T) + 4 * ts + (i & 3); };
+    // a block's offset in its window, the window's first element, the
+    // elements its copy takes (whole packs of kPad), the window element that
+    // slot e stands for and that element's offset from the block's start
+    // (see kPad)
     auto shift = [](int64_t s) { return ODD ? (int)(s & (kPad - 1)) : 0; };
     auto window = [](int64_t s) { return ODD ? s & ~(int64_t)(kPad - 1) : s; };
+    auto span = [&](int64_t s, int l) { return (shift(s) + l + kPad - 1) & ~(kPad - 1); };
     auto welem = [](int e, int sh) { return e < sh ? e + kI8Block : e; };
+    auto woff = [&](int e, int sh) { return welem(e, sh) - sh; };
+    // the window elements [lo, hi) that bulk copies store: all but the ends
+    auto tile_lo = [&](int64_t s) { return shift(s) != 0 ? kPad : 0; };
+    auto tile_hi = [&](int64_t s, int l) {
+        if (!ODD || l == kI8Block) return kI8Block;
+        const int end = (shift(s) + l) & ~(kPad - 1);
+        return end < kI8Block ? end : kI8Block;
+    };
     // a thread's elements of an fp32 array read straight from global memory:
     // 16-byte streaming loads on blocks that move by bulk copies, element
     // loads (0 beyond the block's end) otherwise
@@ -682,9 +701,12 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
         for (int c = 0; c < PER; c += 4) {
             if (whole) {
                 const float *w = src + window(s);
-                if (c == 0 && t < 2 && shift(s) != 0) {
+                if (ODD && (l != kI8Block || (c == 0 && ts < 2 && shift(s) != 0))) {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) o[i] = w[welem(4 * t + i, shift(s))];
+                    for (int i = 0; i < 4; ++i) {
+                        const int e = el(c + i);
+                        o[c + i] = woff(e, shift(s)) < l ? w[welem(e, shift(s))] : 0.f;
+                    }
                     continue;
                 }
                 const float4 q = __ldcs(reinterpret_cast<const float4 *>(w + el(c)));
@@ -696,26 +718,25 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
         }
     };
 
-    // whole blocks whose window lies inside the vector move by bulk copies
-    // (the buffers are 16-byte aligned where a.nvec > 0)
+    // whole aligned blocks move by bulk copies, and in the ODD instances every
+    // block whose window lies inside the vector (the buffers are 16-byte
+    // aligned where a.nvec > 0)
     auto bulk_block = [&](int64_t s, int l) {
         if constexpr (ODD)
-            return l == kI8Block && a.nvec > 0 &&
-                   (shift(s) == 0 || (window(s) >= -a.head && window(s) + kSlot <= a.n));
+            return a.nvec > 0 && window(s) >= -a.head && window(s) + span(s, l) <= a.n;
         else
             return l == kI8Block && a.nvec > 0 && (s % kPad) == 0;
     };
     bool in_flight = false;  // thread 0: bulk loads issued and not yet seen complete
     // thread 0: the bulk copies of group q of the block at s (theta and v
     // come with group 0)
-    auto stage_bulk = [&](int64_t kbi, int64_t s, int q) {
+    auto stage_bulk = [&](int64_t kbi, int64_t s, int l, int q) {
         if (q == 0 && a.test_stall_tile1 != 0 && kbi == a.test_stall_tile1 - 1)
             return;  // testing only: this phase never completes
         const int m0 = q * G;
         const int gq = M - m0 < G ? M - m0 : G;
-        const bool off = shift(s) != 0;
-        const uint32_t gv_bytes = kGVBytes + (off ? kPadGV : 0);
-        const uint32_t x_bytes = kXBytes + (off ? kPadX : 0);
+        const uint32_t gv_bytes = ODD ? span(s, l) * 4 : kGVBytes;
+        const uint32_t x_bytes = ODD ? span(s, l) * ES : kXBytes;
         s = window(s);
         mbar_arrive_expect_tx(bar, (q == 0 && !DGV ? 2 * gv_bytes : 0) + gq * x_bytes);
         if constexpr (PF > 0) {
@@ -745,24 +766,58 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
         }
         in_flight = true;
     };
-    // thread 0 and 1: the wrapped elements of a window that has landed move
-    // into their own slots (group q; theta and v with group 0)
-    auto unwrap = [&](int sh, int q) {
+    // the slots of a window that has landed hold what they stand for: the
+    // wrapped elements (the first chunks) and, in a short block, zeros beyond
+    // its elements, which move no maximum and no sum (group q; theta and v
+    // with group 0).  Every thread settles its own chunks, a chunk at a time.
+    auto settle = [&](int64_t s, int l, int q) {
+        const int sh = shift(s);
         const int m0 = q * G;
         const int gq = M - m0 < G ? M - m0 : G;
-        for (int e = 4 * t; e < 4 * t + 4 && e < sh; ++e) {
-            if (q == 0 && !DGV) {
-                sg[e] = sg[e + kI8Block];
-                sv[e] = sv[e + kI8Block];
+#pragma unroll
+        for (int c = 0; c < PER; c += 4) {
+            if (c > 0 && l == kI8Block) break;
+            const int e0 = el(c);
+            // per element: stays (0), comes from e + 4096 (1), beyond (2)
+            int from[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const bool in = woff(e0 + i, sh) < l;
+                from[i] = in ? (e0 + i >= sh ? 0 : 1) : 2;
             }
-            for (int m = 0; m < gq; ++m) {
-                if constexpr (BF16) {
-                    uint16_t *x = reinterpret_cast<uint16_t *>(sx + m * kXSlot);
-                    x[e] = x[e + kI8Block];
-                } else {
-                    float *x = reinterpret_cast<float *>(sx + m * kXSlot);
-                    x[e] = x[e + kI8Block];
-                }
+            auto pick = [&](int i, auto here, auto there) {
+                return from[i] == 0 ? here : from[i] == 1 ? there : decltype(here)(0);
+            };
+            // the first chunks alone can wrap; others read nothing behind
+            const int e1 = e0 < kPad ? e0 + kI8Block : e0;
+            auto put_f32 = [&](float *p) {
+                const float4 h = *reinterpret_cast<const float4 *>(p + e0);
+                const float4 w = *reinterpret_cast<const float4 *>(p + e1);
+                *reinterpret_cast<float4 *>(p + e0) =
+                    make_float4(pick(0, h.x, w.x), pick(1, h.y, w.y), pick(2, h.z, w.z),
+                                pick(3, h.w, w.w));
+            };
+            auto put_bf16 = [&](uint16_t *p) {
+                const uint2 h = *reinterpret_cast<const uint2 *>(p + e0);
+                const uint2 w = *reinterpret_cast<const uint2 *>(p + e1);
+                auto both = [&](int i, unsigned a, unsigned b) {
+                    return pick(i, a & 0xffffu, b & 0xffffu) |
+                           pick(i + 1, a & 0xffff0000u, b & 0xffff0000u);
+                };
+                *reinterpret_cast<uint2 *>(p + e0) = make_uint2(both(0, h.x, w.x),
+                                                                both(2, h.y, w.y));
+            };
+            if (q == 0 && !DGV) {
+                put_f32(sg);
+                put_f32(sv);
+            }
+#pragma unroll
+            for (int m = 0; m < G; ++m) {
+                if (m >= gq) break;
+                if constexpr (BF16)
+                    put_bf16(reinterpret_cast<uint16_t *>(sx + m * kXSlot));
+                else
+                    put_f32(reinterpret_cast<float *>(sx + m * kXSlot));
             }
         }
         // a later bulk copy overwrites these bytes
@@ -777,9 +832,8 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
         locate_block(P, kbi, ps, pl);
         if (!bulk_block(ps, pl)) return;
         const uint64_t pol = policy_evict_last();
-        const bool off = shift(ps) != 0;
-        const uint32_t gv_bytes = kGVBytes + (off ? kPadGV : 0);
-        const uint32_t x_bytes = kXBytes + (off ? kPadX : 0);
+        const uint32_t gv_bytes = ODD ? span(ps, pl) * 4 : kGVBytes;
+        const uint32_t x_bytes = ODD ? span(ps, pl) * ES : kXBytes;
         ps = window(ps);
         bulk_prefetch_l2_hint(a.g + ps, gv_bytes, pol);
         bulk_prefetch_l2_hint(a.v + ps, gv_bytes, pol);
@@ -788,7 +842,8 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
             bulk_prefetch_l2_hint(reinterpret_cast<const unsigned char *>(a.x[m]) + ps * ES,
                                   x_bytes, pol);
     };
-    // every thread: its own elements of group q of a short or unaligned block
+    // every thread: its own elements of group q of a block that no bulk copy
+    // serves
     auto stage_own = [&](int64_t s, int l, int q) {
         const int m0 = q * G;
         const int gq = M - m0 < G ? M - m0 : G;
@@ -816,11 +871,12 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
         fence_proxy_async_smem();
     };
     // thread 0: the output tiles of the block at s go to global memory
-    // (without the window's ends, which threads 0 and 1 stored)
-    auto store_tiles = [&](int64_t s) {
-        const int skip = shift(s) != 0 ? kPad : 0;
+    // (without the window's ends: store_ends)
+    auto store_tiles = [&](int64_t s, int l) {
+        const int skip = tile_lo(s), count = tile_hi(s, l) - skip;
+        if (ODD && count <= 0) return;
         s = window(s) + skip;
-        const uint32_t gv_bytes = kGVBytes - skip * 4, x_bytes = kXBytes - skip * ES;
+        const uint32_t gv_bytes = count * 4, x_bytes = count * ES;
         const uint32_t from_x = smem_addr(ox) + skip * ES;
         if constexpr (PF > 0) {
             // written once: evict these lines first, ahead of the prefetched ones
@@ -845,6 +901,27 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
         bulk_commit();
     };
 
+    // every warp: the ends of the window at s from the tiles, an array a warp
+    // and an element a lane (lanes 0..7 the first slots, 8..15 what follows
+    // the last whole pack of a short block)
+    auto store_ends = [&](int64_t s, int l) {
+        const int sh = shift(s), hi = tile_hi(s, l);
+        const int e = lane < kPad ? lane : hi + lane - kPad;
+        if (lane >= 2 * kPad || (lane < kPad ? sh == 0 : hi == kI8Block)) return;
+        if (lane >= kPad && e >= sh + l) return;
+        const int off = woff(e, sh);
+        if (off >= l) return;
+        for (int m = warp; m < M + (GV ? 2 : 0); m += W) {
+            if (m >= M)
+                (m == M ? a.g : a.v)[s + off] = (m == M ? og : ov)[e];
+            else if constexpr (BF16)
+                reinterpret_cast<uint16_t *>(a.x[m])[s + off] =
+                    reinterpret_cast<const uint16_t *>(ox)[e];
+            else
+                reinterpret_cast<float *>(a.x[m])[s + off] = og[e];
+        }
+    };
+
     int kb = blockIdx.x;
     int64_t start = 0;
     int len = 0;
@@ -856,7 +933,7 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
         if (!bulk_block(start, len))
             stage_own(start, len, 0);
         else if (t == 0)
-            stage_bulk(kb, start, 0);
+            stage_bulk(kb, start, len, 0);
     }
     int par = 0;
     for (; kb < nblocks; kb += gridDim.x, par ^= 1) {
@@ -885,7 +962,7 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
                 timed_out = !mbar_wait(bar, phase, nullptr);
                 if (t == 0 && !timed_out) in_flight = false;
                 phase ^= 1;
-                if (t < 2 && shift(start) != 0) unwrap(shift(start), 0);
+                if (ODD && (!full || (ts < 2 && shift(start) != 0))) settle(start, len, 0);
             }
 
             if constexpr (!DGV) {
@@ -932,7 +1009,7 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
 #pragma unroll
             for (int m = 0; m < M; m += 2) {
                 RepPair<MIX> xa[NP], xb[NP];
-                staged_reps<M, BF16, T, MIX>(sx, m, t, xa, xb);
+                staged_reps<M, BF16, T, MIX>(sx, m, ts, xa, xb);
                 worker_max(m, xa);
                 if (m + 1 < M) worker_max(m + 1, xb);
             }
@@ -945,7 +1022,8 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
             }
             // every thread wrote its part of the previous block's tiles before
             // the barrier
-            if (pend && t == 0) store_tiles(s_pstart);
+            if (pend && t == 0) store_tiles(s_pstart, s_plen);
+            if (ODD && pend) store_ends(s_pstart, s_plen);
             pend = false;
             {
                 // every warp folds the W warp maxima of each worker (lane w reads
@@ -1001,7 +1079,7 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
             for (int m = 0; m < M; m += 2) {
                 const float4 scr = *reinterpret_cast<const float4 *>(&sr[warp][m]);
                 RepPair<MIX> xa[NP], xb[NP];
-                staged_reps<M, BF16, T, MIX>(sx, m, t, xa, xb);
+                staged_reps<M, BF16, T, MIX>(sx, m, ts, xa, xb);
                 add_worker(make_float2(scr.x, scr.y), xa);
                 if (m + 1 < M) add_worker(make_float2(scr.z, scr.w), xb);
             }
@@ -1019,7 +1097,7 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
                     timed_out = !mbar_wait(bar, phase, nullptr);
                     if (t == 0 && !timed_out) in_flight = false;
                     phase ^= 1;
-                    if (t < 2 && shift(start) != 0) unwrap(shift(start), q);
+                    if (ODD && (!full || (ts < 2 && shift(start) != 0))) settle(start, len, q);
                 }
                 if (q == 0) {
                     if constexpr (!DGV) {
@@ -1066,7 +1144,7 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
                 for (int m = 0; m < G; m += 2) {
                     if (m >= GQ) break;
                     RepPair<MIX> xa[NP], xb[NP];
-                    staged_reps<G, BF16, T, MIX>(sx, m, t, xa, xb, GQ);
+                    staged_reps<G, BF16, T, MIX>(sx, m, ts, xa, xb, GQ);
                     worker_max(m, xa);
                     if (m + 1 < GQ) worker_max(m + 1, xb);
                 }
@@ -1085,7 +1163,8 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
                 if (q == 0) {
                     // every thread wrote its part of the previous block's tiles
                     // before the barrier
-                    if (pend && t == 0) store_tiles(s_pstart);
+                    if (pend && t == 0) store_tiles(s_pstart, s_plen);
+                    if (ODD && pend) store_ends(s_pstart, s_plen);
                     pend = false;
                 }
                 {
@@ -1145,7 +1224,7 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
                     if (m >= GQ) break;
                     const float4 scr = *reinterpret_cast<const float4 *>(&sr[warp][m]);
                     RepPair<MIX> xa[NP], xb[NP];
-                    staged_reps<G, BF16, T, MIX>(sx, m, t, xa, xb, GQ);
+                    staged_reps<G, BF16, T, MIX>(sx, m, ts, xa, xb, GQ);
                     add_worker(make_float2(scr.x, scr.y), xa);
                     if (m + 1 < GQ) add_worker(make_float2(scr.z, scr.w), xb);
                 }
@@ -1154,7 +1233,7 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
                     // next group of the same block goes into them
                     __syncthreads();
                     if (bulk) {
-                        if (t == 0) stage_bulk(kb, start, q + 1);
+                        if (t == 0) stage_bulk(kb, start, len, q + 1);
                     } else {
                         stage_own(start, len, q + 1);
                     }
@@ -1194,18 +1273,20 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
         // (a short or unaligned next block is staged after the stores)
         if constexpr (NEXT_SMEM) {
             if (t == 0 && nk < nblocks && bulk_block(s_nstart[par], s_nlen[par]))
-                stage_bulk(nk, s_nstart[par], 0);
+                stage_bulk(nk, s_nstart[par], s_nlen[par], 0);
         } else if (t == 0 && nk < nblocks) {
             int64_t ns;
             int nl;
             locate_block(P, nk, ns, nl);
-            if (bulk_block(ns, nl)) stage_bulk(nk, ns, 0);
+            if (bulk_block(ns, nl)) stage_bulk(nk, ns, nl, 0);
         }
         // decode, outer step and stores chunk by chunk (4 elements), so a
         // chunk's results alone are live
         const float rs = __frcp_rn(s);
         auto lo_hi = [](const float2 (&p)[2], int i) { return (i & 1) ? p[i >> 1].y : p[i >> 1].x; };
         float2 b2 = splat2(0.f);
+        // a slot's offset from the block's start
+        auto offset = [&](int e) { return ODD && bulk ? woff(e, shift(start)) : e; };
 #pragma unroll
         for (int c = 0; c < PER; c += 4) {
             const int j = c / 2;  // the chunk's first pair
@@ -1225,17 +1306,17 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
             if (!full) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    if (el(c + i) < len) b32 = fmaf(lo_hi(dq, i), lo_hi(dq, i), b32);
+                    if (offset(el(c + i)) < len) b32 = fmaf(lo_hi(dq, i), lo_hi(dq, i), b32);
             }
             if (!(big <= FLT_MAX)) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    if (full || el(c + i) < len) nf += not_finite(lo_hi(gp, i), lo_hi(vp, i));
+                    if (full || offset(el(c + i)) < len)
+                        nf += not_finite(lo_hi(gp, i), lo_hi(vp, i));
             }
 
             // 5. the stores
-            const bool ends = bulk && c == 0 && t < 2 && shift(start) != 0;
-            if (bulk && !ends) {
+            if (bulk) {
                 if constexpr (BF16) {
                     *reinterpret_cast<uint2 *>(ox + el(c) * 2) =
                         make_uint2(pack_bf16x2(gp[0].x, gp[0].y), pack_bf16x2(gp[1].x, gp[1].y));
@@ -1246,7 +1327,17 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
                 if constexpr (GV)
                     *reinterpret_cast<float4 *>(ov + el(c)) =
                         make_float4(vp[0].x, vp[0].y, vp[1].x, vp[1].y);
-                if constexpr (!GV) {
+                if (ODD && !GV &&
+                    (el(c) < tile_lo(start) || el(c) >= tile_hi(start, len))) {
+                    // a window's ends (those of the tiles: store_ends)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int e = offset(el(c + i));
+                        if (e >= len) continue;
+                        a.g[start + e] = lo_hi(gp, i);
+                        a.v[start + e] = lo_hi(vp, i);
+                    }
+                } else if constexpr (!GV) {
                     __stcs(reinterpret_cast<float4 *>(a.g + window(start) + el(c)),
                            make_float4(gp[0].x, gp[0].y, gp[1].x, gp[1].y));
                     __stcs(reinterpret_cast<float4 *>(a.v + window(start) + el(c)),
@@ -1255,8 +1346,7 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
             } else {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    // the element's offset from the block's start
-                    const int e = ends ? welem(el(c + i), shift(start)) - shift(start) : el(c + i);
+                    const int e = offset(el(c + i));
                     if (e >= len) continue;
                     const float gpi = lo_hi(gp, i);
                     a.g[start + e] = gpi;
@@ -1276,7 +1366,10 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
         if (bulk) {
             fence_proxy_async_smem();  // the tiles are read by bulk copies
             pend = true;
-            if (t == 0) s_pstart = start;
+            if (t == 0) {
+                s_pstart = start;
+                s_plen = len;
+            }
         }
         if (nk < nblocks) {
             if constexpr (NEXT_SMEM) {
@@ -1296,7 +1389,8 @@ __global__ void __launch_bounds__(T, (fused_ctas<M, BF16, T>()))
         }
     } else if (pend) {
         __syncthreads();
-        if (t == 0) store_tiles(s_pstart);
+        if (t == 0) store_tiles(s_pstart, s_plen);
+        if (ODD) store_ends(s_pstart, s_plen);
     }
     if (t == 0) bulk_wait_all();
     // the energies still in registers, and the squared means of every block

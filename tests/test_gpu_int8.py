@@ -161,12 +161,13 @@ def test_int8_round_matches_oracle(dt, M, parts_name, form):
                                   ("bf16", 4), ("bf16", 5), ("bf16", 12), ("bf16", 16)])
 def test_blocks_off_a_16_byte_boundary_equal_the_split_form(dt, M, lead):
     """Parts after one of `lead` elements start off a 16-byte boundary, and
-    the fused form stages their whole blocks as windows: for every offset and
+    the fused form stages their blocks as windows: for every offset and
     for theta and v staged and direct, one and two CTAs per SM and worker
     groups, bit for bit the split form, with several blocks to a CTA, short
     blocks between, and a whole last block whose window passes the vector's
     end."""
-    parts = [lead, 700 * 4096 + 5, 2 * 4096, 3, 4096 - lead - 8 + 16, 4096]
+    parts = [lead, 700 * 4096 + 5, 2 * 4096, 3, 1, 2, 7, 8, 9, 16, 17, 4095, 4091, 4088,
+             4096 - lead + 8, 4096]
     w = W.small(sum(parts), M, dt, seed=50 + M)
     sa, _ = schedule_pair(w.schedule)
     outs = []
