@@ -57,12 +57,16 @@ constexpr size_t kTileSmemReserved = 1024;  // reserved by the system per CTA
 
 template <bool BF16>
 __host__ __device__ constexpr int tile_es() { return BF16 ? 2 : 4; }
+// bf16 M = 6, 7: one 512-thread CTA per SM with two stages (see below)
+template <int M, bool BF16>
+__host__ __device__ constexpr bool tile_alone() { return BF16 && (M == 6 || M == 7); }
 // CTAs per SM the shared-memory budget is planned for: 1024 threads per SM
 // (64 registers a thread), except fp32 with M > 8, whose 2048-element stage
-// fits one 512-thread CTA per SM
+// fits one 512-thread CTA per SM, and bf16 M = 6, 7
 template <int M, bool BF16, int T>
 __host__ __device__ constexpr int tile_ctas() {
-    return ALOCO_TILE_CTAS ? ALOCO_TILE_CTAS : (!BF16 && M > 8) ? 1 : 1024 / T;
+    return ALOCO_TILE_CTAS ? ALOCO_TILE_CTAS
+           : (!BF16 && M > 8) || tile_alone<M, BF16>() ? 1 : 1024 / T;
 }
 template <int M, bool BF16, int T>
 __host__ __device__ constexpr size_t tile_budget() {
@@ -95,16 +99,22 @@ __host__ __device__ constexpr bool tile_fit() {
 // 1.4e8 - 5e8 parameters):
 //   fp32: one 1024-thread CTA per SM, 0.96-0.98 for M = 1 and M = 8
 //     against 0.91-0.95 for 256- and 512-thread shapes;
-//   bf16 M <= 4: four 256-thread CTAs per SM with one stage, 0.98 against
-//     0.95-0.97;
+//   bf16 M = 1, 2: one 1024-thread CTA per SM with two stages, 0.97 and 0.965
+//     (1.4e8 parameters; 0.995 and 0.966 at 4e8) against 0.88 and 0.92 (0.905
+//     and 0.945) for four 256-thread CTAs with one;
+//   bf16 M = 3, 4: four 256-thread CTAs per SM with one stage, 0.95-0.98
+//     against 0.91-0.95 for 512 threads with two;
 //   bf16 M >= 5: two 512-thread CTAs per SM with one stage, so that the
-//     fp32 output tiles fit, 0.97-0.98 against 0.93-0.97.
+//     fp32 output tiles fit, 0.97-0.98 against 0.93-0.97; but M = 6, 7: one
+//     such CTA with two stages, 0.987 and 0.978 (0.993 and 0.979 at 4e8)
+//     against 0.950 and 0.967 (0.973 and 0.978).  Three and four stages lose
+//     2-9 % at every bf16 M.
 //   M = 9..16: 512-thread CTAs with one stage (one CTA per SM for fp32,
 //     two for bf16); fp32 0.99-1.00 for M = 12..16 against 0.95-0.97 for
 //     the register pass, bf16 0.96-0.97 for M = 9..12 against 0.955-0.963.
 template <int M, bool BF16>
 __host__ __device__ constexpr int tile_threads_table() {
-    return M > 8 ? 512 : !BF16 ? 1024 : (M <= 4 ? 256 : 512);
+    return M > 8 ? 512 : !BF16 || M <= 2 ? 1024 : (M <= 4 ? 256 : 512);
 }
 // a forced thread count applies where one stage of its blocks fits
 template <int M, bool BF16>
@@ -117,7 +127,8 @@ __host__ __device__ constexpr int tile_threads() {
 template <int M, bool BF16, int T>
 __host__ __device__ constexpr int tile_stages() {
     if (ALOCO_TILE_NS == 1) return 1;
-    const bool two = ALOCO_TILE_NS == 2 || (!BF16 && M <= 8);
+    const bool two =
+        ALOCO_TILE_NS == 2 || (BF16 ? M <= 2 || tile_alone<M, BF16>() : M <= 8);
     return two && tile_fit<M, BF16, T, 2, false>() ? 2 : 1;
 }
 template <int M, bool BF16, int T, int NS>

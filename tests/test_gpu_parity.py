@@ -401,12 +401,13 @@ def test_wide_tile_pass_equals_register_pass_bit_for_bit(N, M, dt):
     assert s1["mean_sq_norm"] == pytest.approx(s2["mean_sq_norm"], rel=RTOL_STAT)
 
 
-@pytest.mark.parametrize("size", [1e-17, 1.0, 5e18])
+@pytest.mark.parametrize("size", [1e-17, 1.0, 2e18])
 @pytest.mark.parametrize("N", [1000, 1_500_001, 11_000_000])
 def test_energies_over_the_whole_float_range(N, size):
     """Energies of tiny and huge pseudo-gradients: a thread's fp32 partial is
     finite, the sums over a warp and a block need not fit a float (small
-    rounds add float pairs, with doubles beyond 2^100)."""
+    rounds add float pairs, with doubles beyond 2^100).  A partial holds at
+    most 64 squares, so the largest size is below sqrt(FLT_MAX / 64) = 2.3e18."""
     w = W.small(N, 1, "f32", seed=5)
     gen = torch.Generator("cuda").manual_seed(N)
     g = torch.zeros(N, device="cuda").normal_(0, size, generator=gen).clamp_(-size, size)
