@@ -214,10 +214,6 @@ __device__ __forceinline__ float codec_code_f(float y, float s, float r) {
     return fminf(fmaxf(t, -127.f), 127.f);
 }
 
-__device__ __forceinline__ int codec_code(float y, float s) {
-    return (int)codec_code_f(y, s, __frcp_rn(s));
-}
-
 // Nearest integer, ties to even, of |t| < 2^22 on the fp32 adder: t + 1.5 *
 // 2^23 has no fraction bits left, so the addition rounds t at the units
 // place (to even on a tie), and subtracting the constant back is exact.
@@ -327,39 +323,5 @@ __device__ __forceinline__ void widen_pairs(const RawPack<BF16> &r, float2 (&o)[
 
 // Workers a round may have (the statistics rows of the reduction).
 constexpr int kMaxI8Workers = 16;
-
-// A replica's raw pack of one thread for any block: the unconditional
-// 16-byte load on full, aligned blocks, element loads (zero beyond the
-// block's end) otherwise.  Zero-filled elements have Delta = 0 and add
-// nothing to a maximum, an energy or a sum.
-template <bool BF16>
-__device__ __forceinline__ RawPack<BF16> load_raw_any(const void *p, int64_t start, int len,
-                                                      bool fast, int t) {
-    if (fast) return load_raw<BF16>(p, start, t);
-    RawPack<BF16> r;
-    if constexpr (BF16) {
-        const uint16_t *h = reinterpret_cast<const uint16_t *>(p) + start;
-        uint32_t w[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int e = 8 * t + 2 * j;
-            const uint32_t lo = e < len ? h[e] : 0u;
-            const uint32_t hi = e + 1 < len ? h[e + 1] : 0u;
-            w[j] = lo | (hi << 16);
-        }
-        r.q[0] = make_uint4(w[0], w[1], w[2], w[3]);
-    } else {
-        const float *f = reinterpret_cast<const float *>(p) + start;
-        float o[kI8PerThread];
-#pragma unroll
-        for (int i = 0; i < kI8PerThread; ++i) {
-            const int e = elem_of<false>(t, i);
-            o[i] = e < len ? f[e] : 0.f;
-        }
-        r.q[0] = make_float4(o[0], o[1], o[2], o[3]);
-        r.q[1] = make_float4(o[4], o[5], o[6], o[7]);
-    }
-    return r;
-}
 
 }  // namespace aloco

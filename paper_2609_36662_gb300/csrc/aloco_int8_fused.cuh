@@ -417,21 +417,6 @@ __device__ __forceinline__ void staged_reps(const unsigned char *sx, int m0, int
     }
 }
 
-// Block-wide max |y| as float bits (NaN, whose bits exceed +inf's, wins):
-// each warp's maximum goes to red[warp]; after the barrier every warp folds
-// the W values with one warp max (lane w reads warp w's value).
-template <int PER, int W>
-__device__ __forceinline__ float block_amax(const float (&y)[PER], unsigned *red) {
-    unsigned m = 0;
-#pragma unroll
-    for (int i = 0; i < PER; ++i) m = max(m, __float_as_uint(fabsf(y[i])));
-    m = __reduce_max_sync(0xffffffffu, m);
-    const int lane = threadIdx.x & 31;
-    if (lane == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    return __uint_as_float(__reduce_max_sync(0xffffffffu, lane < W ? red[lane] : 0u));
-}
-
 // Fewer instructions per element-worker: the block maxima and the codes'
 // half-integer margin taken with three-input maxima, and the exact-quotient
 // fallback as a warp-uniform branch, against two-input maxima, a compare per
@@ -470,7 +455,7 @@ __device__ __forceinline__ float2 code2_fast_max(float2 y, float r, float &far) 
 // Block-wide max |y| of a thread's pairs, as float bits: each warp's
 // maximum goes to red[warp]; after the barrier every warp folds the W values
 // with one warp max.  A NaN wins (the NaN-propagating maximum gives the
-// canonical NaN, whose bits exceed +inf's), as in block_amax.
+// canonical NaN, whose bits exceed +inf's), as block_amax takes it.
 template <int NP, int W>
 __device__ __forceinline__ float block_amax2(const float2 (&y)[NP], unsigned *red) {
     float mf = 0.f;
