@@ -144,8 +144,12 @@ __host__ __device__ constexpr bool tile_gv() {
 // for (two for 32 bf16 workers, one for 32 fp32 workers), with the fp32
 // output tiles.  The register pass at these M holds one 256-thread block per
 // SM, whose loads in flight do not cover HBM latency: 6e6 x 32 bf16 166 us
-// against 151 here (the kernel).
+// against 151 here (the kernel; whole calls 215 and 204, 199 with the grouped
+// loads of single elements).
+// Two CTAs per SM also where three stages would fit (up to 21 bf16 workers): x 20
+// bf16 977 -> 939 us at 6.4e7 parameters, 118 -> 114 at 6e6.
 constexpr int kWideT = 256;
+constexpr int kWideCtas = 2;
 
 template <int MT, bool BF16, int T, int NS>
 __global__ void __launch_bounds__(T, (MT == 0 ? 2 : tile_ctas<MT, BF16, T>()))
@@ -351,17 +355,19 @@ __global__ void __launch_bounds__(T, (MT == 0 ? 2 : tile_ctas<MT, BF16, T>()))
             const float v = a.v[jj];
             float s = 0.f;
 #pragma unroll
-            for (int m = 0; m < MM; ++m) {
-                if (MT == 0 && m >= M) break;
-                float x;
-                if constexpr (BF16)
-                    x = __uint_as_float(
-                        (uint32_t)(reinterpret_cast<const uint16_t *>(a.x[m])[jj]) << 16);
-                else
-                    x = reinterpret_cast<const float *>(a.x[m])[jj];
-                const float d = g - x;
-                s += d;
-                e_acc[m] = fmaf(d, d, e_acc[m]);
+            for (int m0 = 0; m0 < MM; m0 += kElemGroup) {
+                if (MT == 0 && m0 >= M) break;
+                float x[kElemGroup];
+#pragma unroll
+                for (int q = 0; q < kElemGroup; ++q)
+                    if (m0 + q < M) x[q] = load_replica<BF16>(a.x[m0 + q], jj);
+#pragma unroll
+                for (int q = 0; q < kElemGroup; ++q) {
+                    if (m0 + q >= M) continue;
+                    const float d = g - x[q];
+                    s += d;
+                    e_acc[m0 + q] = fmaf(d, d, e_acc[m0 + q]);
+                }
             }
             b32 = fmaf(s, s, b32);
             float gp, vp;
@@ -447,7 +453,7 @@ cudaError_t wide_launch(const SyncArgs &a, int sm_count, int max_grid, cudaStrea
         occ_cache[a.M].set(dev, occ);
     }
     const int64_t nblk = a.n / (4 * kWideT);
-    int64_t grid = (int64_t)sm_count * occ;
+    int64_t grid = (int64_t)sm_count * (occ < kWideCtas ? occ : kWideCtas);
     if (grid > nblk) grid = nblk;
     if (grid > max_grid) grid = max_grid;
     if (grid < 1) grid = 1;
