@@ -547,8 +547,12 @@ class Controller:
 def _parts_array(parts):
     if parts is None:
         return None, 0
-    buf = array.array("q", [int(p) for p in parts])
-    return (ctypes.c_int64 * len(parts)).from_buffer(buf), len(parts)
+    sizes = [int(p) for p in parts]
+    try:
+        arr = (ctypes.c_int64 * len(sizes)).from_buffer(array.array("q", sizes))
+    except OverflowError:  # wraps, and the library refuses what comes of it
+        arr = (ctypes.c_int64 * len(sizes))(*sizes)
+    return arr, len(sizes)
 
 
 def int8_num_blocks(parts) -> int:

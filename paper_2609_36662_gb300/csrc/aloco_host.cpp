@@ -1003,8 +1003,8 @@ int aloco_int8_decode(const int8_t *codes, const float *scales, size_t N,
 // bf16 replicas, whose threads write theta' and v' as two 16-byte halves of
 // 32 bytes, the halves then reach the link apart (161 against 268 GB/s).  Calls,
 // staged (chunks of 2^24) against direct: 1e6 x 4 fp32 227 and 152 us, 5e6 x 4
-// fp32 889 and 622 us, 2e7 x 8 fp32 4461 and 3889 us, the 150M set x 4 bf16 13.0
-// and 12.1 ms (254 and 274 GB/s), x 8 fp32 28.8 and 26.5 ms.
+// fp32 889 and 622 us, 2e7 x 8 fp32 4461 and 3889 us, the 150M set x 4 bf16 12.5
+// and 11.0 ms (265 and 303 GB/s), x 8 fp32 28.0 and 26.5 ms.
 static int host_direct(Workspace *ws, aloco::SyncArgs &a, const aloco_correction_t &corr,
                        aloco_dtype dtype, const aloco_opts_t &o, aloco_stats_t *st) {
     const int M = st->M;
