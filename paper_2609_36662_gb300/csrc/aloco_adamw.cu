@@ -180,6 +180,9 @@ __global__ void __launch_bounds__(kBlock)
         }
     };
     int64_t u0 = (int64_t)blockIdx.x * kBlock + threadIdx.x;
+    // Ahead of the norms: the norm pass let this kernel start only after its
+    // own wait, so everything before it (the last step's update, whoever wrote
+    // x, g, m or v) had completed, and it writes none of these itself.
     if (a.given) wait_for_previous();
     load(u0);
     if (!a.given) wait_for_previous();
@@ -187,7 +190,7 @@ __global__ void __launch_bounds__(kBlock)
         if (threadIdx.x == 0) s_clip = a.clip[m];
     } else if (threadIdx.x < 32) {
         double s = 0.0;
-        for (int b = threadIdx.x; b < a.g1; b += 32) s += a.partials[(int64_t)m * a.g1 + b];
+        for (int b = threadIdx.x; b < a.g1; b += 32) s += __ldcg(a.partials + (int64_t)m * a.g1 + b);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
         if (threadIdx.x == 0) {
