@@ -186,29 +186,14 @@ __device__ __forceinline__ float load_replica(const void *p, int64_t j) {
         return reinterpret_cast<const float *>(p)[j];
 }
 
-// A sum as an unevaluated pair of floats, hi + lo: adding two keeps the
-// rounding error of hi exactly (the two-sum of Knuth, TAOCP 4.2.2) and leaves
-// about 2^-46 of the sum in lo.  Ten fp32 additions, a small part of what
-// one fp64 addition costs here.  hi must not overflow.
-struct FloatPair {
-    float hi, lo;
-};
-__device__ __forceinline__ FloatPair operator+(FloatPair a, FloatPair b) {
-    const float s = __fadd_rn(a.hi, b.hi);
-    const float t = __fsub_rn(s, a.hi);
-    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, t)), __fsub_rn(b.hi, t));
-    return {s, __fadd_rn(__fadd_rn(a.lo, b.lo), e)};
-}
-__device__ __forceinline__ double value(FloatPair a) { return (double)a.hi + (double)a.lo; }
-__device__ __forceinline__ double value(double a) { return a; }
 __device__ __forceinline__ float from_lane_xor(float v, int mask) {
     return __shfl_xor_sync(0xffffffffu, v, mask);
 }
 __device__ __forceinline__ double from_lane_xor(double v, int mask) {
     return __shfl_xor_sync(0xffffffffu, v, mask);
 }
-__device__ __forceinline__ FloatPair from_lane_xor(FloatPair v, int mask) {
-    return {__shfl_xor_sync(0xffffffffu, v.hi, mask), __shfl_xor_sync(0xffffffffu, v.lo, mask)};
+__device__ __forceinline__ unsigned long long from_lane_xor(unsigned long long v, int mask) {
+    return __shfl_xor_sync(0xffffffffu, v, mask);
 }
 
 // Warp sums of the P values each lane holds (P a power of two, at most 32)
@@ -241,6 +226,64 @@ __device__ __forceinline__ T warp_sum_scatter(T (&v)[P]) {
 }
 __host__ __device__ constexpr int pow2_at_least(int n) {
     return n <= 1 ? 1 : 2 * pow2_at_least((n + 1) / 2);
+}
+// Of the P values each lane holds, the one whose warp sum warp_sum_scatter
+// returns there.
+template <int P, typename T>
+__device__ __forceinline__ T lane_value(T (&v)[P]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int n = P, mask = 16; n > 1; n >>= 1, mask >>= 1) {
+        const bool up = (lane & mask) != 0;
+#pragma unroll
+        for (int i = 0; i < n / 2; ++i) v[i] = up ? v[i + n / 2] : v[i];
+    }
+    return v[0];
+}
+
+// Warp sums of non-negative floats as 64-bit integers: a value's mantissa in
+// units of 2^-34 of the last place of the warp's largest value (`top`, its
+// bits), so that 32 of them fit and add without rounding.  A value below 2^-34
+// of the largest loses less than a unit, 2^-57 of the largest, and the
+// conversion at the end rounds once: at most 31 x 2^-57 + 2^-53 of the sum, where
+// the five roundings of a sum of doubles leave up to 5 x 2^-53.  An addition is two
+// integer ones, where an fp64 one holds the SM's fp64 pipe for 16 clocks.
+// An infinity or NaN comes back from `top` itself.
+__device__ __forceinline__ unsigned warp_top(float e) {
+    return __reduce_max_sync(0xffffffffu, __float_as_uint(e));
+}
+__device__ __forceinline__ unsigned long long to_fixed(float e, unsigned top) {
+    // biased exponents; a subnormal has the smallest normal one
+    const int ee = max((int)(__float_as_uint(e) >> 23), 1);
+    const int et = max((int)(top >> 23), 1);
+    const unsigned mant = __float_as_uint(e) - ((unsigned)(ee - 1) << 23);
+    return ((unsigned long long)mant << 34) >> min(et - ee, 63);
+}
+__device__ __forceinline__ double from_fixed(unsigned long long sum, unsigned top) {
+    if (top >= 0x7f800000u) return (double)__uint_as_float(top);
+    const int et = max((int)(top >> 23), 1);
+    // times 2^(et - 184)
+    return __ull2double_rn(sum) * __hiloint2double((1023 + et - 184) << 20, 0);
+}
+// Lane L returns the sum over the warp of value L >> (5 - log2 P).
+template <int P>
+__device__ __forceinline__ double warp_sum_scatter_exact(const float (&e)[P]) {
+    unsigned top[P];
+    unsigned long long v[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+        top[i] = warp_top(e[i]);
+        v[i] = to_fixed(e[i], top[i]);
+    }
+    const unsigned long long sum = warp_sum_scatter<P>(v);
+    return from_fixed(sum, lane_value<P>(top));
+}
+__device__ __forceinline__ double warp_sum_exact(float e) {
+    const unsigned top = warp_top(e);
+    unsigned long long v = to_fixed(e, top);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += from_lane_xor(v, off);
+    return from_fixed(v, top);
 }
 // The sum of column `col` over rows 0..n - 1 (n <= 32), in every lane.
 template <int COLS>
@@ -364,26 +407,41 @@ __device__ __forceinline__ void finish_rows(const SyncArgs &a, int M, double (&r
     }
 }
 
-// The same from per-thread fp64 partials, folded across each warp first:
-// the energies by recursive halving (about MM adds a warp instead of 5 MM).
-// Against shuffle trees over every value in every thread, serial folds in one
-// thread and a serial publish: 2^20 parameters x 4 fp32 workers 20.0 -> 15.1
-// us (the kernel, ncu), 6e6 x 32 bf16 190 -> 166 us; the fused INT8 kernel, 1024
-// threads a block, 2e7 x 16 bf16 385 -> 300 us, 2e7 x 8 fp32 330 -> 283 us.  S bounds the rows where shared memory is short.
-template <int MM, typename T>
-__device__ __forceinline__ void fold_warp(double (&row)[MM + 1], const T (&e)[MM], T b) {
+// A warp's row from its threads' partials: energies by recursive halving
+// (about MM additions a warp instead of 5 MM), in doubles or, from fp32
+// partials, in fixed point.
+template <int MM>
+__device__ __forceinline__ void store_row(double (&row)[MM + 1], double energy, double b) {
     constexpr int P = pow2_at_least(MM);
-    const int lane = threadIdx.x & 31;
-    T v[P];
-#pragma unroll
-    for (int m = 0; m < P; ++m) v[m] = m < MM ? e[m < MM ? m : 0] : T{};
-    const double sum = value(warp_sum_scatter<P>(v));
-    const int w = lane / (32 / P);
-    if (lane % (32 / P) == 0 && w < MM) row[w] = sum;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) b = b + from_lane_xor(b, off);
-    if (lane == 0) row[MM] = value(b);
+    const int lane = threadIdx.x & 31, m = lane / (32 / P);
+    if (lane % (32 / P) == 0 && m < MM) row[m] = energy;
+    if (lane == 0) row[MM] = b;
 }
+template <int MM>
+__device__ __forceinline__ void fold_warp(double (&row)[MM + 1], const double (&e)[MM], double b) {
+    constexpr int P = pow2_at_least(MM);
+    double v[P];
+#pragma unroll
+    for (int m = 0; m < P; ++m) v[m] = m < MM ? e[m < MM ? m : 0] : 0.0;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) b += from_lane_xor(b, off);
+    store_row<MM>(row, warp_sum_scatter<P>(v), b);
+}
+template <int MM>
+__device__ __forceinline__ void fold_warp(double (&row)[MM + 1], const float (&e)[MM], float b) {
+    constexpr int P = pow2_at_least(MM);
+    float v[P];
+#pragma unroll
+    for (int m = 0; m < P; ++m) v[m] = m < MM ? e[m < MM ? m : 0] : 0.f;
+    store_row<MM>(row, warp_sum_scatter_exact<P>(v), warp_sum_exact(b));
+}
+
+// finish_rows from per-thread fp64 partials.  Against shuffle trees over
+// every value in every thread, serial folds in one thread and a serial
+// publish: 2^20 parameters x 4 fp32 workers 20.0 -> 15.1 us (the kernel, ncu),
+// 6e6 x 32 bf16 190 -> 166 us; the fused INT8 kernel, 1024 threads a block,
+// 2e7 x 16 bf16 385 -> 300 us, 2e7 x 8 fp32 330 -> 283 us.  S bounds the rows
+// where shared memory is short.
 template <int MM, int NW, int S = 32>
 __device__ __forceinline__ void reduce_and_finish(const SyncArgs &a, int M,
                                                   double (&e64)[MM], double b64,
@@ -575,22 +633,14 @@ __global__ void __launch_bounds__(kBlock, (min_blocks<MT, BF16>()))
         }
     }
     // A small round: no thread has come to a flush, so its sums are the fp32
-    // partials, and a warp adds them as float pairs instead of doubles (which
-    // took 3 to 5 us of a round: the flush and the warp's sums, with the fp64
-    // pipe of an SM at two additions a clock; the kernel at 2^20 parameters: 8 fp32
-    // workers 22.5 -> 18.1 us, 4 16.8 -> 14.5, 16 bf16 25.0 -> 22.9).  Partials above 2^100, whose
-    // pair could overflow, infinities and NaN take the doubles.
+    // partials, and a warp adds them in fixed point instead of doubles (the
+    // flush and the warp's sums took 3 to 5 us of a round, with the fp64 pipe
+    // of an SM at two additions a clock).
     const int64_t loose = a.head + a.n - a.nvec * PACK;
     const bool small = (a.nvec + stride - 1) / stride + (loose + stride - 1) / stride < kFlush;
-    float top = b32;
-#pragma unroll
-    for (int m = 0; m < MM; ++m) top = e32[m] <= 0x1p100f ? top : e32[m];
     __shared__ double rows[32][MM + 1];
-    if (small && __all_sync(0xffffffffu, top <= 0x1p100f)) {
-        FloatPair pairs[MM];
-#pragma unroll
-        for (int m = 0; m < MM; ++m) pairs[m] = {e32[m], 0.f};
-        fold_warp<MM>(rows[threadIdx.x >> 5], pairs, FloatPair{b32, 0.f});
+    if (small) {
+        fold_warp<MM>(rows[threadIdx.x >> 5], e32, b32);
     } else {
         flush();
         fold_warp<MM>(rows[threadIdx.x >> 5], e64, b64);

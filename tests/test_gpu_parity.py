@@ -406,8 +406,8 @@ def test_wide_tile_pass_equals_register_pass_bit_for_bit(N, M, dt):
 def test_energies_over_the_whole_float_range(N, size):
     """Energies of tiny and huge pseudo-gradients: a thread's fp32 partial is
     finite, the sums over a warp and a block need not fit a float (small
-    rounds add float pairs, with doubles beyond 2^100).  A partial holds at
-    most 64 squares, so the largest size is below sqrt(FLT_MAX / 64) = 2.3e18."""
+    rounds add the partials in fixed point).  A partial holds at most 64
+    squares, so the largest size is below sqrt(FLT_MAX / 64) = 2.3e18."""
     w = W.small(N, 1, "f32", seed=5)
     gen = torch.Generator("cuda").manual_seed(N)
     g = torch.zeros(N, device="cuda").normal_(0, size, generator=gen).clamp_(-size, size)
@@ -418,6 +418,43 @@ def test_energies_over_the_whole_float_range(N, size):
     assert st["status"] == A.OK
     assert st["D"] == pytest.approx(energy, rel=RTOL_STAT)
     assert st["mean_sq_norm"] == pytest.approx(energy, rel=RTOL_STAT)
+
+
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+@pytest.mark.parametrize("M", [1, 2, 8, 16, 32])
+def test_small_round_energies_are_summed_without_rounding(M, dt):
+    """Energies that a double holds exactly come out exactly: each thread's
+    partial is one odd 24-bit square, one thread's is 2^52, and their sums
+    need up to 53 bits."""
+    pack = 4 if dt == "f32" else 8
+    N = 256 * pack
+    w = W.small(N, M, dt, seed=3)
+    g = torch.zeros(N, device="cuda")
+    g[::pack] = 4095.0
+    g[5 * pack] = 2.0 ** 26
+    energy = 2.0 ** 52 + 255 * 4095.0 ** 2
+    v = torch.zeros(N, device="cuda")
+    xs = [torch.zeros(N, dtype=torch.float32 if dt == "f32" else torch.bfloat16, device="cuda")
+          for _ in range(M)]
+    st = run_gpu_round(g, v, xs, w, w.start_step, w.H_sel[0])
+    assert st["status"] == A.OK
+    assert st["drift"] == [energy] * M
+    assert st["mean_sq_norm"] == energy
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_small_round_reports_nonfinite_energies(bad):
+    """The energy of a replica with an infinity is infinite, with a NaN a NaN;
+    the other replicas' energies are untouched."""
+    N = 3000
+    g = torch.ones(N, device="cuda")
+    v = torch.zeros(N, device="cuda")
+    xs = [torch.zeros(N, device="cuda") for _ in range(3)]
+    xs[1][1234] = bad
+    w = W.small(N, 3, "f32", seed=3)
+    st = run_gpu_round(g, v, xs, w, w.start_step, w.H_sel[0])
+    assert st["status"] == A.ERR_NONFINITE
+    np.testing.assert_equal(st["drift"], [float(N), bad, float(N)])
 
 
 def test_auto_pass_choice():
