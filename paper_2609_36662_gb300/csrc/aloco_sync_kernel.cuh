@@ -265,13 +265,17 @@ __device__ __forceinline__ double from_fixed(unsigned long long sum, unsigned to
     // times 2^(et - 184)
     return __ull2double_rn(sum) * __hiloint2double((1023 + et - 184) << 20, 0);
 }
-// Lane L returns the sum over the warp of value L >> (5 - log2 P).
+// Lane L returns the sum over the warp of value L >> (5 - log2 P); values
+// from `used` on are 0 (`used` is the same in every lane).
 template <int P>
-__device__ __forceinline__ double warp_sum_scatter_exact(const float (&e)[P]) {
+__device__ __forceinline__ double warp_sum_scatter_exact(const float (&e)[P], int used = P) {
     unsigned top[P];
     unsigned long long v[P];
 #pragma unroll
     for (int i = 0; i < P; ++i) {
+        top[i] = 0;
+        v[i] = 0;
+        if (i >= used) continue;
         top[i] = warp_top(e[i]);
         v[i] = to_fixed(e[i], top[i]);
     }

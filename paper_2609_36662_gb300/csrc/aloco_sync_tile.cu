@@ -26,8 +26,8 @@
 // have read their tiles, so block j + 1 may rewrite them.
 // Elements after the last whole block are handled element by element.
 // Drift energies sum in fp32 per thread over at most 8 blocks (32 squares)
-// before each warp adds them, in a fixed order, to its fp64 row; the
-// statistics agree with the register pass within the statistics tolerance.
+// before each warp adds them, in a fixed order, to its fp64 row (M > 16: see
+// kWideFlushBlocks); the statistics agree with the register pass within the statistics tolerance.
 #include "aloco_bulk.cuh"
 #include "aloco_sync_kernel.cuh"
 
@@ -148,8 +148,15 @@ __host__ __device__ constexpr bool tile_gv() {
 // loads of single elements).
 // Two CTAs per SM also where three stages would fit (up to 21 bf16 workers): x 20
 // bf16 977 -> 939 us at 6.4e7 parameters, 118 -> 114 at 6e6.
+// The warps add their threads' energies in fixed point, no less exactly
+// than the register pass in doubles, every 16 blocks: a thread's partial then
+// holds 64 squares, as the register pass's for fp32 replicas (128 for bf16).
+// Against fp32 warp sums every 8 blocks (with events, L2 flushed): 6e6 x 32
+// bf16 156.3 us both, 6.4e7 x 17 bf16 850.6 -> 854.7 us, 6.4e7 x 32 fp32
+// 2590 -> 2594 us.
 constexpr int kWideT = 256;
 constexpr int kWideCtas = 2;
+constexpr int kWideFlushBlocks = 16;
 
 template <int MT, bool BF16, int T, int NS>
 __global__ void __launch_bounds__(T, (MT == 0 ? 2 : tile_ctas<MT, BF16, T>()))
@@ -185,7 +192,7 @@ __global__ void __launch_bounds__(T, (MT == 0 ? 2 : tile_ctas<MT, BF16, T>()))
     auto flush = [&]() {
         if constexpr (MT == 0) {
             // lane m gets worker m's warp sum
-            e_w[warp][lane] += (double)warp_sum_scatter<MM>(e_acc);
+            e_w[warp][lane] += warp_sum_scatter_exact<MM>(e_acc, M);
 #pragma unroll
             for (int m = 0; m < MM; ++m) e_acc[m] = 0.f;
         } else {
@@ -332,7 +339,7 @@ __global__ void __launch_bounds__(T, (MT == 0 ? 2 : tile_ctas<MT, BF16, T>()))
             if constexpr (!GV) stcs4(a.g + e, 0, make_float4(gp[0], gp[1], gp[2], gp[3]));
         }
         fence_proxy_async_smem();  // the tiles are read by bulk copies
-        if (++since_flush == kTileFlushBlocks) flush();
+        if (++since_flush == (MT == 0 ? kWideFlushBlocks : kTileFlushBlocks)) flush();
         b64 += (double)b32;
         b32 = 0.f;
     }

@@ -421,6 +421,48 @@ def test_energies_over_the_whole_float_range(N, size):
 
 
 @pytest.mark.parametrize("dt", ["f32", "bf16"])
+@pytest.mark.parametrize("M", [17, 32])
+@pytest.mark.parametrize("size", [1e-17, 1.0, 2e18])
+def test_wide_tile_energies_over_the_whole_float_range(size, M, dt):
+    """As above through the tile pass, 16 blocks (64 squares) to a partial.
+    Replicas at 0 and at 2 theta in turn keep the summed pseudo-gradient at
+    0 or theta."""
+    N = (1 << 24) + 1000
+    w = W.small(N, M, dt, seed=6)
+    tdt = torch.float32 if dt == "f32" else torch.bfloat16
+    gen = torch.Generator("cuda").manual_seed(M)
+    g = torch.zeros(N, device="cuda").normal_(0, size, generator=gen).clamp_(-size, size)
+    g = g.bfloat16().float()  # 2 theta is then exact in either type
+    v = torch.zeros(N, device="cuda")
+    xs = [(2 * g if m % 2 else torch.zeros_like(g)).to(tdt) for m in range(M)]
+    energy = float(g.double().square().sum())
+    st = run_gpu_round(g, v, xs, w, w.start_step, w.H_sel[0])
+    assert (st["status"], st["pass_used"]) == (A.OK, A.PASS_TILE)
+    np.testing.assert_allclose(st["drift"], [energy] * M, rtol=RTOL_STAT)
+    assert st["mean_sq_norm"] == pytest.approx(energy * (M % 2) / M ** 2, rel=RTOL_STAT)
+
+
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+@pytest.mark.parametrize("M", [17, 32])
+def test_wide_tile_energies_are_summed_without_rounding(M, dt):
+    """Partials of up to 16 odd squares below 2^24 and one of 2^52: their
+    warps' and blocks' sums fit a double and come out exactly."""
+    N = 1 << 22
+    w = W.small(N, M, dt, seed=6)
+    g = torch.zeros(N, device="cuda")
+    g[::4] = 1023.0
+    g.view(-1, 1024)[:, :4] = 0.0  # one thread's elements, but the one
+    g[0] = 2.0 ** 26
+    energy = 2.0 ** 52 + N // 1024 * 255 * 1023.0 ** 2
+    v = torch.zeros(N, device="cuda")
+    xs = [torch.zeros(N, dtype=torch.float32 if dt == "f32" else torch.bfloat16, device="cuda")
+          for _ in range(M)]
+    st = run_gpu_round(g, v, xs, w, w.start_step, w.H_sel[0])
+    assert (st["status"], st["pass_used"]) == (A.OK, A.PASS_TILE)
+    assert st["drift"] == [energy] * M
+
+
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
 @pytest.mark.parametrize("M", [1, 2, 8, 16, 32])
 def test_small_round_energies_are_summed_without_rounding(M, dt):
     """Energies that a double holds exactly come out exactly: each thread's
