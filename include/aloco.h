@@ -278,8 +278,9 @@ int aloco_sync_ex(float *global, float *momentum, void *const *locals,
 
 /* One outer round (as aloco_sync_ex, Algorithm 1) on state that lives in
  * host memory: theta, v and the M replicas are page-locked host arrays
- * (cudaMallocHost, or registered with cudaHostRegister); any other memory
- * is ALOCO_ERR_ARG.  With chunk_elems = 0 and buffers that reach a 16-byte
+ * (cudaMallocHost, or registered with cudaHostRegister) over their whole
+ * length; any other memory is ALOCO_ERR_ARG.  With chunk_elems = 0 and
+ * buffers that each lie in one page-locked allocation and reach a 16-byte
  * boundary at the same element, one kernel reads and writes them over the
  * host link, without staging.  Otherwise the library streams them through
  * cached device staging in chunks of chunk_elems elements (0 = 2^24; rounded

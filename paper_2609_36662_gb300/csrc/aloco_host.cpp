@@ -995,6 +995,32 @@ int aloco_int8_decode(const int8_t *codes, const float *scales, size_t N,
     return ALOCO_OK;
 }
 
+// The first address in [p, p + bytes) that is not page-locked (0: none), p
+// itself being so.  *one stays true where the driver places the range in one
+// allocation: memory locked in several pieces, or whose extent the driver does
+// not tell, is for the copies of the staged round to judge.
+static uintptr_t page_locked_gap(uintptr_t p, size_t bytes, bool *one) {
+    const GetAddressRangeFn fn = address_range_fn();
+    for (uintptr_t at = p; at < p + bytes;) {
+        if (at != p) {
+            *one = false;
+            cudaPointerAttributes a;
+            const cudaError_t e = cudaPointerGetAttributes(&a, (const void *)at);
+            if (e != cudaSuccess) cudaGetLastError();
+            if (e != cudaSuccess || a.type != cudaMemoryTypeHost) return at;
+        }
+        CUdeviceptr base = 0;
+        size_t size = 0;
+        if (!fn || fn(&base, &size, (CUdeviceptr)at) != CUDA_SUCCESS ||
+            (uintptr_t)base + size <= at) {
+            *one = false;
+            return 0;
+        }
+        at = (uintptr_t)base + size;
+    }
+    return 0;
+}
+
 // The host-memory round without staging: the register pass on the buffers'
 // device addresses, the replicas read only.  The host link bounds it, and the
 // loads and stores of one kernel keep both directions of the link busy from
@@ -1107,23 +1133,26 @@ int aloco_sync_host(float *global, float *momentum, const void *const *locals,
     for (int m = 0; m < M; ++m)
         if ((uintptr_t)locals[m] & (rsz - 1))
             return fail(ALOCO_ERR_ARG, "locals[%d] not %zu-byte aligned", m, rsz);
-    bool mapped = false;  // every buffer has a device address
+    // every buffer has a device address and lies in one page-locked allocation
+    bool mapped = true;
     void *dev_ptrs[2 + ALOCO_MAX_WORKERS];
-    {
-        const void *ptrs[2 + ALOCO_MAX_WORKERS] = {global, momentum};
-        for (int m = 0; m < M; ++m) ptrs[2 + m] = locals[m];
-        mapped = true;
-        for (int i = 0; i < M + 2; ++i) {
-            cudaPointerAttributes at;
-            cudaError_t e = cudaPointerGetAttributes(&at, ptrs[i]);
-            if (e != cudaSuccess) cudaGetLastError();
-            if (e != cudaSuccess || at.type != cudaMemoryTypeHost)
-                return fail(ALOCO_ERR_ARG,
-                            "buffer %d is not page-locked host memory (allocate it with "
-                            "cudaMallocHost or register it with cudaHostRegister)", i);
-            dev_ptrs[i] = at.devicePointer;
-            mapped = mapped && at.devicePointer;
-        }
+    for (int i = 0; i < M + 2; ++i) {
+        const void *p = i == 0 ? global : i == 1 ? momentum : locals[i - 2];
+        const size_t bytes = N * (i < 2 ? 4 : rsz);
+        cudaPointerAttributes at;
+        cudaError_t e = cudaPointerGetAttributes(&at, p);
+        if (e != cudaSuccess) cudaGetLastError();
+        if (e != cudaSuccess || at.type != cudaMemoryTypeHost)
+            return fail(ALOCO_ERR_ARG,
+                        "buffer %d is not page-locked host memory (allocate it with "
+                        "cudaMallocHost or register it with cudaHostRegister)", i);
+        const uintptr_t gap = page_locked_gap((uintptr_t)p, bytes, &mapped);
+        if (gap)
+            return fail(ALOCO_ERR_ARG,
+                        "buffer %d: of %zu bytes from %p, those from %p on are not "
+                        "page-locked host memory", i, bytes, p, (void *)gap);
+        dev_ptrs[i] = at.devicePointer;
+        mapped = mapped && at.devicePointer;
     }
     size_t chunk = chunk_elems ? chunk_elems : ((size_t)1 << 24);
     chunk = (chunk + 7) / 8 * 8;

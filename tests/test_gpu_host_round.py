@@ -148,3 +148,67 @@ def test_host_round_on_views(off, off_v, dt, chunk):
         assert torch.equal(_bits(whole), _bits(before))
     assert st_h["D"] == pytest.approx(st_d["D"], rel=RTOL_STAT)
     assert st_h["C"] == pytest.approx(st_d["C"], rel=RTOL_STAT)
+
+
+def _on_pages(t, pages):
+    """A copy of the CPU vector t that starts on a 64 KB page of ordinary
+    memory, `pages` of them, and the address of the first."""
+    whole = torch.full(((pages + 1) * 65536 // t.element_size(),), 3.5, dtype=t.dtype)
+    skip = (-whole.data_ptr() % 65536) // t.element_size()
+    part = whole[skip:skip + t.numel()]
+    part.copy_(t)
+    return whole, part
+
+
+@pytest.mark.parametrize("chunk", [0, 4096])
+@pytest.mark.parametrize("short", [0, 1, 3])
+def test_memory_locked_in_part_is_rejected(short, chunk):
+    """A buffer (theta, v, a replica) whose page-locked range ends before the
+    vector does is refused before anything is launched or written."""
+    w = W.small(40_000, 3, "f32", seed=2)   # 160,000 bytes: 2.4 pages of 64 KB
+    g, v, xs = gpu_inputs(w)
+    bufs = [_pinned(t) for t in (g, v, *xs)]
+    whole, part = _on_pages(bufs[short], 3)
+    cudart = torch.cuda.cudart()
+    assert int(cudart.cudaHostRegister(part.data_ptr(), 65536, 0)) == 0
+    try:
+        bufs[short] = part
+        before = [b.clone() for b in bufs]
+        sa, _ = schedule_pair(w.schedule)
+        with pytest.raises(A.AlocoError) as ei:
+            A.sync_host(bufs[0], bufs[1], bufs[2:], H_sel=w.H_sel[0], H_base=w.H_base,
+                        step=w.start_step, schedule=sa, outer_lr=w.outer_lr,
+                        outer_beta=w.outer_beta, chunk_elems=chunk)
+        assert ei.value.status == A.ERR_ARG and "page-locked" in str(ei.value)
+        assert all(torch.equal(b, c) for b, c in zip(bufs, before))
+    finally:
+        assert int(cudart.cudaHostUnregister(part.data_ptr())) == 0
+
+
+def test_memory_locked_in_pieces_is_staged():
+    """Buffers page-locked in pieces, with chunks that end where the pieces do:
+    copied piece by piece."""
+    N = 3 * 16384
+    w = W.small(N, 2, "f32", seed=2)
+    g, v, xs = gpu_inputs(w)
+    v.normal_(0, 1e-3, generator=torch.Generator("cuda").manual_seed(2))
+    pages = [_on_pages(t.cpu(), 3) for t in (g, v, *xs)]
+    cudart = torch.cuda.cudart()
+    pieces = [part.data_ptr() + 65536 * k for _, part in pages for k in range(3)]
+    locked = []
+    try:
+        for p in pieces:
+            assert int(cudart.cudaHostRegister(p, 65536, 0)) == 0
+            locked.append(p)
+        sa, _ = schedule_pair(w.schedule)
+        kw = dict(H_sel=w.H_sel[0], H_base=w.H_base, step=w.start_step, schedule=sa,
+                  outer_lr=w.outer_lr, outer_beta=w.outer_beta)
+        A.sync(g, v, xs, **kw)
+        st = A.sync_host(pages[0][1], pages[1][1], [p for _, p in pages[2:]],
+                         chunk_elems=16384, **kw)
+        assert st["status"] == A.OK and st["grid"] == 3   # chunks
+        assert torch.equal(_bits(pages[0][1]), _bits(g.cpu()))
+        assert torch.equal(_bits(pages[1][1]), _bits(v.cpu()))
+    finally:
+        for p in locked:
+            assert int(cudart.cudaHostUnregister(p)) == 0
