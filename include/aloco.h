@@ -282,7 +282,9 @@ int aloco_sync_ex(float *global, float *momentum, void *const *locals,
  * length; any other memory is ALOCO_ERR_ARG.  With chunk_elems = 0 and
  * buffers that each lie in one page-locked allocation and reach a 16-byte
  * boundary at the same element, one kernel reads and writes them over the
- * host link, without staging.  Otherwise the library streams them through
+ * host link, without staging, on a part of the SMs (opts->blocks_per_sm = k:
+ * k blocks on every SM, which slow other streams' kernels down far more).
+ * Otherwise the library streams them through
  * cached device staging in chunks of chunk_elems elements (0 = 2^24; rounded
  * up to a multiple of 8), overlapping the host-to-device copy of one chunk,
  * the fused kernel on another and the device-to-host copy of theta' and v' of

@@ -1021,16 +1021,38 @@ static uintptr_t page_locked_gap(uintptr_t p, size_t bytes, bool *one) {
     return 0;
 }
 
+// Blocks of the host-memory round without staging.  Loads from host memory
+// take some microseconds, and a block that waits for them holds its SM's load
+// units: with one block on every SM, work on other streams ran 2 to 14 times
+// slower during the round (bf16 8192^3 matrix products beside 6e7 x 16 bf16
+// 8.7x, beside 1.2e7 x 32 7.4x; 1 GB additions beside the 150M set x 4 bf16
+// 2.0x; 4 MB ones 3 to 14x).  The link needs about 0.6 MB in flight, so no more
+// blocks run than hold kHostInFlight, and at least three sixteenths of the SMs
+// (28 of 152; 64 blocks for one fp32 worker).
+// Rounds with 152, 38, 28 and 19 blocks: 150M x 4 bf16 (128 bytes a thread) 10.94,
+// 10.93, 10.94 and 11.02 ms, 3e7 x 2 bf16 (96) 1.85, 1.85, 1.85 and 2.02 ms, 6e7 x
+// 1 fp32 (48) 3.66, 3.80, 4.42 and 5.55 ms (64 blocks 3.66), 2e7 x 8 fp32 3.88 ms
+// each; from 5e4 parameters on no count is faster than these.  Counts that are
+// no multiple of 4 lost 1-4 % (25 blocks: 11.06 ms, 6e7 x 16 bf16 12.04 against
+// 11.56 ms).
+constexpr size_t kHostInFlight = 768 << 10;
+static int host_blocks(int M, aloco_dtype dtype, int sm_count) {
+    const int pack = aloco::pack_elems(dtype);
+    const size_t block = (size_t)aloco::kBlock * (8 * pack + 16 * M);
+    const int need = (int)((kHostInFlight + block - 1) / block);
+    return std::max((need + 3) / 4 * 4, std::max(sm_count * 3 / 16 / 4 * 4, 4));
+}
+
 // The host-memory round without staging: the register pass on the buffers'
 // device addresses, the replicas read only.  The host link bounds it, and the
 // loads and stores of one kernel keep both directions of the link busy from
 // the first pack to the last, where staged chunks copy in before anything
-// computes and out after it.  One block per SM: more gain nothing, and with
-// bf16 replicas, whose threads write theta' and v' as two 16-byte halves of
-// 32 bytes, the halves then reach the link apart (161 against 268 GB/s).  Calls,
-// staged (chunks of 2^24) against direct: 1e6 x 4 fp32 227 and 152 us, 5e6 x 4
-// fp32 889 and 622 us, 2e7 x 8 fp32 4461 and 3889 us, the 150M set x 4 bf16 12.5
-// and 11.0 ms (265 and 303 GB/s), x 8 fp32 28.0 and 26.5 ms.
+// computes and out after it.  At most one block per SM: with more, and bf16
+// replicas, whose threads write theta' and v' as two 16-byte halves of 32
+// bytes, the halves reach the link apart (161 against 268 GB/s).  Calls,
+// staged (chunks of 2^24) against direct: 2e5 x 4 fp32 91 and 51 us, 1e6 x 4 217
+// and 145 us, 3e6 x 4 543 and 381 us, 2e7 x 8 fp32 4385 and 3880 us, 6e7 x 16 bf16 12.7
+// and 11.6 ms, the 150M set x 4 bf16 12.45 and 10.94 ms (265 and 302 GB/s).
 static int host_direct(Workspace *ws, aloco::SyncArgs &a, const aloco_correction_t &corr,
                        aloco_dtype dtype, const aloco_opts_t &o, aloco_stats_t *st) {
     const int M = st->M;
@@ -1052,6 +1074,8 @@ static int host_direct(Workspace *ws, aloco::SyncArgs &a, const aloco_correction
     cudaError_t e = dtype == ALOCO_F32
                         ? aloco::plan_sync_f32(M, a.nvec, ws->sm_count, bps, &plan)
                         : aloco::plan_sync_bf16(M, a.nvec, ws->sm_count, bps, &plan);
+    if (o.blocks_per_sm == 0)
+        plan.grid = std::min(plan.grid, host_blocks(M, dtype, ws->sm_count));
     if (e != cudaSuccess) return cuda_fail(e, "launch plan");
     cudaStream_t stream = (cudaStream_t)o.stream;
     if (o.time_kernel) e = cudaEventRecord(ws->ev0, stream);

@@ -212,3 +212,23 @@ def test_memory_locked_in_pieces_is_staged():
     finally:
         for p in locked:
             assert int(cudart.cudaHostUnregister(p)) == 0
+
+
+@pytest.mark.parametrize("dt,M", [("f32", 1), ("f32", 8), ("bf16", 1), ("bf16", 32)])
+def test_host_round_leaves_most_sms_to_other_streams(dt, M):
+    """The round without staging runs on less than half of the SMs unless the
+    caller asks for blocks on every one; the results do not depend on it."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    w = W.small(1_000_003, M, dt, seed=12)
+    g, v, xs = gpu_inputs(w)
+    sa, _ = schedule_pair(w.schedule)
+    kw = dict(H_sel=w.H_sel[0], H_base=w.H_base, step=w.start_step, schedule=sa,
+              outer_lr=w.outer_lr, outer_beta=w.outer_beta)
+    outs = []
+    for opts in (A.default_opts(), A.default_opts(blocks_per_sm=1)):
+        gh, vh, xh = _pinned(g), _pinned(v), [_pinned(x) for x in xs]
+        outs.append((A.sync_host(gh, vh, xh, opts=opts, **kw), gh, vh))
+    (a, ga, va), (b, gb, vb) = outs
+    assert a["grid"] < sms / 2 and b["grid"] == sms
+    assert torch.equal(ga, gb) and torch.equal(va, vb)
+    assert a["D"] == pytest.approx(b["D"], rel=RTOL_STAT)
