@@ -121,7 +121,8 @@ typedef enum {
  *   AUTO       the fastest as measured on GB300 for (M, dtype, N): TILE
  *              from 2^27 parameters for bf16 replicas with M <= 12 and for
  *              fp32 with M = 1 or 5..16, and from 2^22 parameters for M > 16
- *              (aligned buffers), else REGISTERS.
+ *              (aligned buffers, blocks_per_sm = 0), else REGISTERS.  A TILE
+ *              request for M > 16 still runs REGISTERS.
  * The INT8-communicated round (aloco_sync_int8) has two forms of its own:
  *   INT8_SPLIT a block-scale kernel, then an apply kernel that reads the
  *              replicas again (any M <= 16);
@@ -172,7 +173,7 @@ typedef struct aloco_opts {
     int32_t mode;         /* aloco_corr_mode                                 */
     int32_t time_kernel;  /* 1: stats_out->kernel_ms = duration of the fused
                              pass, from CUDA events on the launch stream     */
-    int32_t blocks_per_sm;/* resident blocks per SM of the fused pass; 0 =
+    int32_t blocks_per_sm;/* resident blocks per SM of the register pass; 0 =
                              the library's tuned choice for (M, dtype).  It
                              is capped at what the kernel's registers allow.
                              The grid fixes the order of the fp64 partial

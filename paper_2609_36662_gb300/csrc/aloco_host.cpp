@@ -362,7 +362,8 @@ bool use_int8_fused(int pass, int M, aloco_dtype dtype) {
 }
 
 
-bool use_tile(int pass, int M, aloco_dtype dtype, int64_t n, int64_t nvec) {
+bool use_tile(int pass, int M, aloco_dtype dtype, int64_t n, int64_t nvec,
+              int blocks_per_sm) {
     if (!sync_tile_fits(M, n, nvec)) return false;
     if (pass == ALOCO_PASS_TILE) return M <= 16;
     if (pass != ALOCO_PASS_AUTO) return false;
@@ -371,7 +372,7 @@ bool use_tile(int pass, int M, aloco_dtype dtype, int64_t n, int64_t nvec) {
     // copy peak, x 17 0.72 against 0.62, 6.4e7 x 32 bf16 0.96 against 0.85, fp32
     // 0.99 against 0.84; at 2e6 they tie for bf16, and fp32 with 24 and 32
     // workers is 4-7 % slower.
-    if (M > 16) return n >= (1 << 22);
+    if (M > 16) return n >= (1 << 22) && blocks_per_sm == 0;
     // AUTO, as measured on GB300 (fraction of the measured copy peak): from
     // 2^27 parameters the tile pass leads for bf16 replicas (0.97-0.98
     // against 0.94) and for fp32 with M = 1 or M >= 5 (0.96-0.98 against
@@ -694,7 +695,7 @@ int sync_impl(float *global, float *momentum, void *const *locals, size_t N,
     aloco::LaunchPlan plan;
     // the staged passes take aligned buffers; the register pass serves a head
     const int64_t staged = a.head == 0 ? a.nvec : 0;
-    const bool tile = !int8 && aloco::use_tile(o.pass, M, dtype, a.n, staged);
+    const bool tile = !int8 && aloco::use_tile(o.pass, M, dtype, a.n, staged, o.blocks_per_sm);
     const bool tma = !int8 && !tile && aloco::use_tma(o.pass, M, dtype, staged);
     const bool fused = int8 && aloco::use_int8_fused(o.pass, M, dtype);
     if (fused || tile) {

@@ -119,9 +119,11 @@ cudaError_t plan_sync_tma_bf16(int M, int64_t nvec, int sm_count,
 bool use_tma(int pass, int M, aloco_dtype dtype, int64_t nvec);
 // The tile pass (aloco_sync_tile.cu): aligned buffers, at least one whole
 // block.  An explicit TILE request serves M <= 16; AUTO takes it for more
-// workers too.
+// workers too, unless blocks_per_sm asks for a residency, which the register
+// pass alone has.
 bool sync_tile_fits(int M, int64_t n, int64_t nvec);
-bool use_tile(int pass, int M, aloco_dtype dtype, int64_t n, int64_t nvec);
+bool use_tile(int pass, int M, aloco_dtype dtype, int64_t n, int64_t nvec,
+              int blocks_per_sm);
 cudaError_t launch_sync_tile(const SyncArgs &a, aloco_dtype dtype, int sm_count,
                              int max_grid, cudaStream_t stream, int *grid_out);
 // Whether an INT8 round of M workers (dtype) uses the fused form.

@@ -190,7 +190,7 @@ extern "C" int aloco_sync_noalloc(float *global, float *momentum,
     aloco::LaunchPlan plan;
     // the same choice of kernel as aloco_sync_ex
     const int64_t staged = a.head == 0 ? a.nvec : 0;
-    const bool tile = aloco::use_tile(o.pass, M, dtype, a.n, staged);
+    const bool tile = aloco::use_tile(o.pass, M, dtype, a.n, staged, o.blocks_per_sm);
     const bool tma = !tile && aloco::use_tma(o.pass, M, dtype, staged);
     plan.grid = 0;
     plan.block = 0;

@@ -401,6 +401,20 @@ def test_wide_tile_pass_equals_register_pass_bit_for_bit(N, M, dt):
     assert s1["mean_sq_norm"] == pytest.approx(s2["mean_sq_norm"], rel=RTOL_STAT)
 
 
+@pytest.mark.parametrize("noalloc", [False, True])
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+def test_auto_honours_blocks_per_sm_above_16_workers(dt, noalloc):
+    """A residency that the caller asks for is the register pass's."""
+    w = W.small(1 << 22, 17, dt, seed=17)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    g, v, xs = gpu_inputs(w)
+    st = A.sync(g, v, xs, H_sel=w.H_sel[0], H_base=w.H_base, step=w.start_step,
+                schedule=schedule_pair(w.schedule)[0], outer_lr=w.outer_lr,
+                outer_beta=w.outer_beta, opts=A.default_opts(blocks_per_sm=1),
+                noalloc=noalloc)
+    assert (st["status"], st["pass_used"], st["grid"]) == (A.OK, A.PASS_REGISTERS, sms)
+
+
 @pytest.mark.parametrize("size", [1e-17, 1.0, 2e18])
 @pytest.mark.parametrize("N", [1000, 1_500_001, 11_000_000])
 def test_energies_over_the_whole_float_range(N, size):
