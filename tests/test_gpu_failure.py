@@ -169,3 +169,70 @@ def test_stalled_int8_worker_group_block_is_reported_and_the_device_stays_usable
     for a_, b_ in zip(x1, x2):
         assert torch.equal(a_.view(torch.int32), b_.view(torch.int32))
 
+
+
+@pytest.mark.parametrize("M,dt", [(17, "bf16"), (32, "bf16"), (32, "f32")])
+def test_stalled_wide_tile_block_is_reported_and_the_device_stays_usable(M, dt):
+    """The tile pass above 16 workers (two CTAs per SM; 32 fp32 workers: one)."""
+    w = W.small(1 << 22, M, dt, seed=5)
+    kw = _kw(w)
+    g, v, xs = gpu_inputs(w)
+    st = A.sync(g, v, xs, **kw)
+    assert st["status"] == A.OK and st["pass_used"] == A.PASS_TILE
+    block = 3 * st["grid"] + 11            # the fourth block of CTA 11
+    assert block < w.numel // 1024
+
+    g, v, xs = gpu_inputs(w)
+    A.test_stall_tile(block)
+    t0 = time.time()
+    st = A.sync(g, v, xs, raise_on_error=False, **kw)
+    took = time.time() - t0
+    assert st["status"] == A.ERR_CUDA
+    assert "timed out" in A.last_error()
+    assert 1.0 < took < 60.0, took
+    torch.cuda.synchronize()
+
+    g1, v1, x1 = gpu_inputs(w)
+    g2, v2, x2 = gpu_inputs(w)
+    st1 = A.sync(g1, v1, x1, **kw)
+    st2 = A.sync(g2, v2, x2, opts=A.default_opts(pass_=A.PASS_REGISTERS), **kw)
+    assert st1["status"] == st2["status"] == A.OK
+    assert st1["pass_used"] == A.PASS_TILE
+    assert torch.equal(g1, g2) and torch.equal(v1, v2)
+    assert all(torch.equal(a, b) for a, b in zip(x1, x2))
+
+
+@pytest.mark.parametrize("M,dt", [(4, "bf16"), (16, "bf16"), (12, "f32")],
+                         ids=["two_ctas", "one_cta_prefetch", "worker_groups"])
+@pytest.mark.parametrize("short", [False, True], ids=["whole", "short"])
+def test_stalled_int8_window_is_reported_and_the_device_stays_usable(short, M, dt):
+    """The fused INT8 round on blocks off a 16-byte boundary: a window of a
+    whole or of a short block that never arrives."""
+    # codec block k > 0: whole ones of one part, or the short ones of 800 parts
+    parts = [5, 1 << 22] if not short else [5] + [1501] * 800 + [1 << 21]
+    w = W.small(sum(parts), M, dt, seed=6)
+    kw = dict(_kw(w), parts=parts)
+    fused = lambda: A.default_opts(pass_=A.PASS_INT8_FUSED)
+    g, v, xs = gpu_inputs(w)
+    st = A.sync_int8(g, v, xs, opts=fused(), **kw)
+    assert st["status"] == A.OK and st["pass_used"] == A.PASS_INT8_FUSED
+    block = st["grid"] + 9                  # the second block of CTA 9
+    assert block < 800
+
+    g, v, xs = gpu_inputs(w)
+    A.test_stall_tile(block)
+    t0 = time.time()
+    st = A.sync_int8(g, v, xs, opts=fused(), raise_on_error=False, **kw)
+    took = time.time() - t0
+    assert st["status"] == A.ERR_CUDA
+    assert "timed out" in A.last_error()
+    assert 1.0 < took < 60.0, took
+    torch.cuda.synchronize()
+
+    g1, v1, x1 = gpu_inputs(w)
+    g2, v2, x2 = gpu_inputs(w)
+    st1 = A.sync_int8(g1, v1, x1, opts=fused(), **kw)
+    st2 = A.sync_int8(g2, v2, x2, opts=A.default_opts(pass_=A.PASS_INT8_SPLIT), **kw)
+    assert st1["status"] == st2["status"] == A.OK
+    assert torch.equal(g1, g2) and torch.equal(v1, v2)
+    assert all(torch.equal(a, b) for a, b in zip(x1, x2))
