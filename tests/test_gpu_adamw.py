@@ -227,3 +227,77 @@ def test_normed_step_matches_the_oracle():
     orc = _oracle(xs, gs, m1, m2, O.F32, O.F32, cfg)
     st = A.adamw_step(xs, gs, m1, m2, A.adamw_cfg(**cfg), grad_norms=orc["norms"])
     _compare(xs, m1, m2, st, orc, O.F32)
+
+
+def _produce(bufs, k):
+    """A backward pass's stand-in, on the current stream: gradients and
+    parameters change in place, and so do the moments once."""
+    xs, gs, m1, m2 = bufs
+    for x, g in zip(xs, gs):
+        g.mul_(-0.75).add_(x, alpha=0.01)
+        x.mul_(1.0 - 2.0 ** -10)
+    if k == 1:
+        for a, b in zip(m1, m2):
+            a.neg_()
+            b.mul_(1.5)
+
+
+@pytest.mark.parametrize("given", [False, True], ids=["norm_pass", "given_norms"])
+@pytest.mark.parametrize("N,M,dt,steps", [(5, 1, O.F32, 40), (3001, 3, O.BF16, 40),
+                                          (300_007, 4, O.F32, 20), (5_000_008, 4, O.BF16, 6),
+                                          (9_000_003, 2, O.F32, 6)])
+def test_queued_steps_and_producers_equal_synchronised_ones(N, M, dt, steps, given):
+    """The update starts while the norm pass runs and loads before it waits
+    for the norms: steps queued right behind kernels that write their
+    parameters, gradients and moments equal, bit for bit, the same sequence
+    with a wait after every kernel.  From one block to several waves."""
+    cfg = A.adamw_cfg(**dict(C4, lr=4e-3, step=9))
+    norms = dict(grad_norms=[0.5 + m for m in range(M)]) if given else {}
+    side = torch.cuda.Stream()
+    results = []
+    for wait in (True, False):
+        bufs = _state(N, M, dt, dt, seed=21)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            for k in range(steps):
+                _produce(bufs, k)
+                if wait:
+                    side.synchronize()
+                A.adamw_step(*bufs, cfg, want_stats=False, **norms)
+                if wait:
+                    side.synchronize()
+        side.synchronize()
+        results.append(bufs)
+    for a, b in zip(sum(results[0], []), sum(results[1], [])):
+        assert torch.equal(a, b)
+
+
+def test_captured_steps_equal_eager_ones():
+    """Under capture the step follows a memory set, a kernel and a join with
+    another stream, and a second step follows the first."""
+    cfg = A.adamw_cfg(**dict(C4, lr=4e-3, step=9))
+
+    def body(bufs, other):
+        xs, gs, m1, m2 = bufs
+        main = torch.cuda.current_stream()
+        other.wait_stream(main)
+        with torch.cuda.stream(other):
+            for x, g in zip(xs, gs):
+                g.add_(x, alpha=0.125)
+        m1[0].zero_()
+        main.wait_stream(other)
+        A.adamw_step(*bufs, cfg, want_stats=False)
+        A.adamw_step(*bufs, cfg, want_stats=False)
+
+    eager, captured = (_state(200_003, 3, O.F32, O.BF16, seed=22) for _ in range(2))
+    other = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    A.adamw_step(*_state(1000, 1, O.F32, O.BF16, seed=1), cfg)  # the workspace exists
+    with torch.cuda.graph(graph):
+        body(captured, other)
+    for _ in range(5):
+        graph.replay()
+        body(eager, other)
+    torch.cuda.synchronize()
+    for a, b in zip(sum(eager, []), sum(captured, [])):
+        assert torch.equal(a, b)
