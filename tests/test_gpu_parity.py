@@ -515,18 +515,27 @@ def test_small_round_reports_nonfinite_energies(bad):
 
 def test_auto_pass_choice():
     """AUTO runs the tile pass from 2^27 parameters for fp32 with M = 1 or
-    5..16 and for bf16 with M <= 12, and the register pass elsewhere (fp32
-    M = 2..4, bf16 M >= 13, smaller rounds).  The buffers are zeros: only
-    the choice is checked."""
-    big, small = (1 << 27) + 4096, (1 << 27) - 4096
+    5..16 and for bf16 with M <= 12, from 2^22 for M > 16, and the register
+    pass elsewhere (fp32 M = 2..4, bf16 M = 13..16, smaller rounds, views that
+    start off a 16-byte boundary).  The buffers are zeros: only the choice is
+    checked."""
+    big, small, wide = (1 << 27) + 4096, (1 << 27) - 4096, 1 << 22
     sched = A.Schedule.make()
     cases = [(big, 8, torch.float32, A.PASS_TILE), (big, 1, torch.float32, A.PASS_TILE),
              (big, 3, torch.float32, A.PASS_REGISTERS), (big, 4, torch.bfloat16, A.PASS_TILE),
-             (big, 13, torch.bfloat16, A.PASS_REGISTERS), (small, 8, torch.float32, A.PASS_REGISTERS)]
-    for n, M, dt, want in cases:
-        g = torch.zeros(n, device="cuda")
-        v = torch.zeros(n, device="cuda")
-        xs = [torch.zeros(n, dtype=dt, device="cuda") for _ in range(M)]
+             (big, 13, torch.bfloat16, A.PASS_REGISTERS), (small, 8, torch.float32, A.PASS_REGISTERS),
+             (wide, 17, torch.float32, A.PASS_TILE), (wide, 32, torch.bfloat16, A.PASS_TILE),
+             (wide - 1, 17, torch.float32, A.PASS_REGISTERS),
+             (wide - 1, 32, torch.bfloat16, A.PASS_REGISTERS),
+             (wide, 16, torch.float32, A.PASS_REGISTERS),
+             (wide, 16, torch.bfloat16, A.PASS_REGISTERS)]
+    heads = [(wide + 64, 24, torch.float32, A.PASS_REGISTERS),
+             (wide + 64, 24, torch.bfloat16, A.PASS_REGISTERS)]
+    for n, M, dt, want in cases + heads:
+        skip = 3 if (n, M, dt, want) in heads else 0
+        g = torch.zeros(n + skip, device="cuda")[skip:]
+        v = torch.zeros(n + skip, device="cuda")[skip:]
+        xs = [torch.zeros(n + skip, dtype=dt, device="cuda")[skip:] for _ in range(M)]
         st = A.sync(g, v, xs, H_sel=150, H_base=100, step=4000, schedule=sched,
                     outer_lr=0.7, outer_beta=0.9)
         assert st["status"] == A.OK and st["pass_used"] == want, (n, M, dt, st["pass_used"])
