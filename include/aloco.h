@@ -147,7 +147,7 @@ typedef enum {
  * the shard calls):
  *   SPIN   the calling thread polls the device-mapped page that the round's
  *          last block publishes its statistics to, checking the stream every
- *          few hundred reads.  Lowest latency (the call returns a few
+ *          few thousand reads.  Lowest latency (the call returns a few
  *          microseconds after the last block), but the thread keeps one host
  *          core busy for the whole round, including any time the stream is
  *          queued behind earlier work.

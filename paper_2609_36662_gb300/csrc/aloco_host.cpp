@@ -368,10 +368,17 @@ bool use_tile(int pass, int M, aloco_dtype dtype, int64_t n, int64_t nvec,
     if (pass == ALOCO_PASS_TILE) return M <= 16;
     if (pass != ALOCO_PASS_AUTO) return false;
     // M = 17..32, against the register pass (one block per SM, whose loads in
-    // flight do not cover HBM latency): 6e6 x 32 bf16 0.77 against 0.73 of the
-    // copy peak, x 17 0.72 against 0.62, 6.4e7 x 32 bf16 0.96 against 0.85, fp32
-    // 0.99 against 0.84; at 2e6 they tie for bf16, and fp32 with 24 and 32
-    // workers is 4-7 % slower.
+    // flight do not cover HBM latency, but whose first packs come sooner).  The
+    // line is where the tile pass leads at every M and type; it is about 2^20
+    // to 2^21 at 17 workers and 2^21 to 2^22 at 24 and more.  Kernel us, L2
+    // flushed, registers then tile, fp32 / bf16:
+    //   1e6    x 17   45.7  43.6 /  33.4  34.8   x 32   63.4  69.3 /  44.7  49.8
+    //   2e6    x 17   73.9  68.2 /  49.8  46.7   x 24   87.7  90.7 /  55.9  58.0
+    //          x 28  101.0 101.0 /  64.1  64.1   x 32  110.2 111.2 /  68.2  70.3
+    //   3e6    x 24  131.7 123.5 /  73.7  74.4   x 32  164.5 152.2 /  92.6  92.3
+    //   4.2e6  x 17  144.0 119.4 /  84.6  76.4   x 24  174.7 159.9 /  98.9  94.8
+    //          x 32  221.8 196.3 / 123.5 119.4
+    //   6.4e7  x 17   1834  1552 /  1014   850   x 32   3043  2585 /  1603  1391
     if (M > 16) return n >= (1 << 22) && blocks_per_sm == 0;
     // AUTO, as measured on GB300 (fraction of the measured copy peak): from
     // 2^27 parameters the tile pass leads for bf16 replicas (0.97-0.98
