@@ -1040,9 +1040,11 @@ static uintptr_t page_locked_gap(uintptr_t p, size_t bytes, bool *one) {
 // Rounds with 152, 38, 28 and 19 blocks: 150M x 4 bf16 (128 bytes a thread) 10.94,
 // 10.93, 10.94 and 11.02 ms, 3e7 x 2 bf16 (96) 1.85, 1.85, 1.85 and 2.02 ms, 6e7 x
 // 1 fp32 (48) 3.66, 3.80, 4.42 and 5.55 ms (64 blocks 3.66), 2e7 x 8 fp32 3.88 ms
-// each; from 5e4 parameters on no count is faster than these.  Counts that are
-// no multiple of 4 lost 1-4 % (25 blocks: 11.06 ms, 6e7 x 16 bf16 12.04 against
-// 11.56 ms).
+// each; from 5e4 parameters on no count is faster than these.  How the blocks'
+// strides fall on a buffer's pages moves single counts by 1-4 % (25 blocks:
+// 11.06 ms, 6e7 x 16 bf16 12.04 against 11.56 ms; in another call 36 blocks: 11.11
+// ms); 28 stayed within 0.5 % of 152.  Counts are multiples of 4, of which fewer
+// were moved.
 constexpr size_t kHostInFlight = 768 << 10;
 static int host_blocks(int M, aloco_dtype dtype, int sm_count) {
     const int pack = aloco::pack_elems(dtype);
