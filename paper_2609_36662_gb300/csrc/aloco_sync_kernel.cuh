@@ -173,11 +173,6 @@ struct Pack<true> {
     }
 };
 
-// Replica values of one element that are loaded before any is used, in the
-// loops over single elements: with the worker count known only at run time,
-// the loads otherwise wait for one another (at the end of a round of 6e6 x 32
-// bf16 this took 12 us, and takes 4).
-constexpr int kElemGroup = 16;
 template <bool BF16>
 __device__ __forceinline__ float load_replica(const void *p, int64_t j) {
     if constexpr (BF16)
@@ -595,23 +590,30 @@ __global__ void __launch_bounds__(kBlock, (min_blocks<MT, BF16>()))
     // where the buffers share no 16-byte boundary.  A call on one of three
     // shards of 5e7 x 6 bf16, cut off a boundary, took 267 us element by
     // element and takes 144 us with its packs behind a head.
+    // With the worker count known only at run time the loads go out 16 at a
+    // time and whatever the count (replica 0 again beyond it): behind a test of
+    // the count each waits for the one before.  Whole vectors element by
+    // element (kernel), tested one by one, tested in groups of 16, and this: 1.6e7
+    // x 17 bf16 1010, 1359 and 644 us, x 32 1076, 1942 and 723; fp32 x 17 935, 1100
+    // and 689, x 32 1109, 1326 and 930.
     constexpr int PACK = BF16 ? 8 : 4;
     for (int64_t r = tid; r < a.head + a.n - a.nvec * PACK; r += stride) {
         const int64_t j = r < a.head ? r - a.head : a.nvec * PACK + r - a.head;
         const float g = a.g[j];
         const float v = a.v[j];
         float s = 0.f;
+        constexpr int kElemGroup = BF16 && MT > 0 ? MT : 16;
 #pragma unroll
         for (int m0 = 0; m0 < MM; m0 += kElemGroup) {
-            if (MT == 0 && m0 >= M) break;
             float x[kElemGroup];
 #pragma unroll
             for (int q = 0; q < kElemGroup; ++q)
-                if (m0 + q < M) x[q] = load_replica<BF16>(a.x[m0 + q], j);
+                if (MT == 0 || m0 + q < M)
+                    x[q] = load_replica<BF16>(a.x[m0 + q < M ? m0 + q : 0], j);
 #pragma unroll
             for (int q = 0; q < kElemGroup; ++q) {
-                if (m0 + q >= M) continue;
-                const float d = g - x[q];
+                if (MT > 0 && m0 + q >= M) continue;
+                const float d = m0 + q < M ? g - x[q] : 0.f;
                 s += d;
                 e32[m0 + q] = fmaf(d, d, e32[m0 + q]);
             }
