@@ -151,9 +151,8 @@ __host__ __device__ constexpr bool tile_gv() {
 // The warps add their threads' energies in fixed point, no less exactly
 // than the register pass in doubles, every 16 blocks: a thread's partial then
 // holds 64 squares, as the register pass's for fp32 replicas (128 for bf16).
-// Against fp32 warp sums every 8 blocks (with events, L2 flushed): 6e6 x 32
-// bf16 156.3 us both, 6.4e7 x 17 bf16 850.6 -> 854.7 us, 6.4e7 x 32 fp32
-// 2590 -> 2594 us.
+// Against fp32 warp sums every 8 blocks this takes about 1 us a round: 4.2e6 x
+// 17 bf16 76.5 -> 77.9 us, 6e6 x 32 156.3 -> 157.1, 2.4e7 x 32 fp32 987.6 -> 988.2.
 constexpr int kWideT = 256;
 constexpr int kWideCtas = 2;
 constexpr int kWideFlushBlocks = 16;
@@ -260,6 +259,7 @@ __global__ void __launch_bounds__(T, (MT == 0 ? 2 : tile_ctas<MT, BF16, T>()))
         for (int64_t j = 0; j < issued; ++j) issue(j);
     }
     bool failed = false;
+    bool loose = false;  // an element after the last whole block was this thread's
     for (int64_t j = 0; j < mine; ++j) {
         const int s = (int)(j % NS);
         const unsigned char *st = smem + (size_t)s * kStage;
@@ -361,6 +361,10 @@ __global__ void __launch_bounds__(T, (MT == 0 ? 2 : tile_ctas<MT, BF16, T>()))
             const float g = a.g[jj];
             const float v = a.v[jj];
             float s = 0.f;
+            // replica values loaded before any is used: an element or none is
+            // left for a thread, whose loads otherwise wait for one another
+            // (at the end of a round of 6e6 x 32 bf16 12 us one by one, 4 now)
+            constexpr int kElemGroup = 16;
 #pragma unroll
             for (int m0 = 0; m0 < MM; m0 += kElemGroup) {
                 if (MT == 0 && m0 >= M) break;
@@ -376,6 +380,7 @@ __global__ void __launch_bounds__(T, (MT == 0 ? 2 : tile_ctas<MT, BF16, T>()))
                     e_acc[m0 + q] = fmaf(d, d, e_acc[m0 + q]);
                 }
             }
+            loose = true;
             b32 = fmaf(s, s, b32);
             float gp, vp;
             outer_step(k, s, g, v, gp, vp);
@@ -392,8 +397,9 @@ __global__ void __launch_bounds__(T, (MT == 0 ? 2 : tile_ctas<MT, BF16, T>()))
             }
         }
     }
+    // (not once more after a flush of the last block)
+    if (MT > 0 || since_flush > 0 || __any_sync(0xffffffffu, loose)) flush();
     if (t == 0) bulk_wait_all();
-    flush();
     b64 += (double)b32;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) b64 += __shfl_down_sync(0xffffffffu, b64, off);
