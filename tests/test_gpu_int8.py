@@ -186,6 +186,34 @@ def test_blocks_off_a_16_byte_boundary_equal_the_split_form(dt, M, lead):
     np.testing.assert_allclose(sta["C"], stb["C"], rtol=RTOL_STAT)
 
 
+@pytest.mark.parametrize("blocks,odd_blocks", [(801, 1), (2431, 1), (2432, 1), (2432, 152),
+                                               (2432, 153), (3000, 700)])
+@pytest.mark.parametrize("M", [8, 9, 12, 13])
+def test_few_blocks_off_a_boundary_equal_the_split_form(M, blocks, odd_blocks):
+    """9 to 12 bf16 workers take up to a sixteenth of the blocks element by
+    element in vectors of 16 blocks per SM (2432 of 152 SMs) and more, and as
+    windows otherwise: bit for bit the split form."""
+    lead = blocks // 2
+    parts = [lead * 4096, 3, odd_blocks * 4096 - 3, (blocks - lead - odd_blocks - 2) * 4096 + 17]
+    assert sum((p + 4095) // 4096 for p in parts) == blocks
+    w = W.small(sum(parts), M, "bf16", seed=50 + M)
+    outs = []
+    for form in ("split", "fused"):
+        g, v, xs = gpu_inputs(w)
+        v.normal_(0, 1e-3, generator=torch.Generator("cuda").manual_seed(M))
+        st = A.sync_int8(g, v, xs, parts=parts, H_sel=w.H_sel[0], H_base=w.H_base,
+                         step=w.start_step, schedule=schedule_pair(w.schedule)[0],
+                         outer_lr=w.outer_lr, outer_beta=w.outer_beta,
+                         opts=A.default_opts(pass_=FORMS[form]))
+        assert st["status"] == A.OK and st["pass_used"] == FORMS[form]
+        outs.append((st, g, v, xs))
+    (sta, ga, va, xa), (stb, gb, vb, xb) = outs
+    assert torch.equal(ga, gb) and torch.equal(va, vb)
+    assert all(torch.equal(p, q) for p, q in zip(xa, xb))
+    np.testing.assert_allclose(sta["drift"], stb["drift"], rtol=RTOL_STAT)
+    np.testing.assert_allclose(sta["C"], stb["C"], rtol=RTOL_STAT)
+
+
 @pytest.mark.parametrize("dt,M", [("f32", 1), ("f32", 4), ("f32", 7), ("bf16", 2),
                                   ("bf16", 5), ("bf16", 8), ("bf16", 9), ("bf16", 12),
                                   ("bf16", 16), ("f32", 9), ("f32", 12), ("f32", 16)])
