@@ -1034,23 +1034,19 @@ static uintptr_t page_locked_gap(uintptr_t p, size_t bytes, bool *one) {
 // units: with one block on every SM, work on other streams ran 2 to 14 times
 // slower during the round (bf16 8192^3 matrix products beside 6e7 x 16 bf16
 // 8.7x, beside 1.2e7 x 32 7.4x; 1 GB additions beside the 150M set x 4 bf16
-// 2.0x; 4 MB ones 3 to 14x).  The link needs about 0.6 MB in flight, so no more
-// blocks run than hold kHostInFlight, and at least three sixteenths of the SMs
-// (28 of 152; 64 blocks for one fp32 worker).
-// Rounds with 152, 38, 28 and 19 blocks: 150M x 4 bf16 (128 bytes a thread) 10.94,
-// 10.93, 10.94 and 11.02 ms, 3e7 x 2 bf16 (96) 1.85, 1.85, 1.85 and 2.02 ms, 6e7 x
-// 1 fp32 (48) 3.66, 3.80, 4.42 and 5.55 ms (64 blocks 3.66), 2e7 x 8 fp32 3.88 ms
-// each; from 5e4 parameters on no count is faster than these.  How the blocks'
-// strides fall on a buffer's pages moves single counts by 1-4 % (25 blocks:
-// 11.06 ms, 6e7 x 16 bf16 12.04 against 11.56 ms; in another call 36 blocks: 11.11
-// ms); 28 stayed within 0.5 % of 152.  Counts are multiples of 4, of which fewer
-// were moved.
+// 2.0x; 4 MB ones 3 to 14x).  The link needs about 0.6 MB in flight: what
+// kHostInFlight takes, and at least a third of the SMs, which no box was seen
+// to need more than.  Rounds with 152, 64, 48, 38, 28 and 24 blocks: 150M x 4 bf16
+// (128 bytes a thread) 10.95, 10.94, 10.93, 10.94, 11.26 and 11.00 ms on one GPU,
+// 10.94, 10.94, 10.94, 10.97, 10.95 and 10.96 on another; 5e7 x 12 bf16 7.78, 7.75,
+// 7.75, 7.76, 8.03 and 8.14 ms; 2e7 x 1 fp32 (48 bytes a thread) 1.24, 1.25, 1.25,
+// 1.30 and 1.53 ms with 28; from 5e4 parameters on no count is faster than these.
 constexpr size_t kHostInFlight = 768 << 10;
 static int host_blocks(int M, aloco_dtype dtype, int sm_count) {
     const int pack = aloco::pack_elems(dtype);
     const size_t block = (size_t)aloco::kBlock * (8 * pack + 16 * M);
     const int need = (int)((kHostInFlight + block - 1) / block);
-    return std::max((need + 3) / 4 * 4, std::max(sm_count * 3 / 16 / 4 * 4, 4));
+    return std::max((need + 7) / 8 * 8, std::max(sm_count / 3 / 8 * 8, 8));
 }
 
 // The host-memory round without staging: the register pass on the buffers'
