@@ -285,11 +285,12 @@ int aloco_sync_ex(float *global, float *momentum, void *const *locals,
  * boundary at the same element, one kernel reads and writes them over the
  * host link, without staging, on a part of the SMs (opts->blocks_per_sm = k:
  * k blocks on every SM, which slow other streams' kernels down far more).
- * Otherwise the library streams them through
- * cached device staging in chunks of chunk_elems elements (0 = 2^24; rounded
- * up to a multiple of 8), overlapping the host-to-device copy of one chunk,
- * the fused kernel on another and the device-to-host copy of theta' and v' of
- * a third, on two internal copy streams and opts->stream.
+ * Otherwise the library streams them through cached device staging in chunks
+ * of chunk_elems elements (0 = 2^24; rounded up to a multiple of 8),
+ * overlapping the host-to-device copy of one chunk, the fused kernel on
+ * another and the device-to-host copy of theta' and v' of a third, on two
+ * internal copy streams and opts->stream: slower, but the SMs are free but for
+ * the short kernels.
  *   global, momentum  in: theta, v; out: theta', v' (fp32, N each);
  *   locals            in only: the replicas' endpoints.  The host replicas
  *                     are NOT reset; the reset replicas equal theta', which
