@@ -155,6 +155,64 @@ def test_views_at_one_offset_equal_aligned_buffers(N, offset, dt, int8):
     assert a["C"] == pytest.approx(b["C"], rel=1e-6)
 
 
+@pytest.mark.parametrize("nan", [False, True])
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+@pytest.mark.parametrize("M", [17, 24, 31, 32])
+@pytest.mark.parametrize("N", [5, 1000, 150_001])
+def test_element_path_above_16_workers_equals_aligned_buffers(N, M, dt, nan):
+    """Buffers at differing offsets go element by element, with replica 0 read
+    in the place of the workers beyond M: bit for bit the aligned round, and a
+    NaN in replica 0 reaches no other energy."""
+    w = W.small(N, M, dt, seed=M)
+    g, v, xs = gpu_inputs(w)
+    if nan:
+        xs[0][3] = float("nan")
+    whole = [torch.full((N + 8,), 3.5, dtype=t.dtype, device="cuda") for t in (g, v, *xs)]
+    views = [t[k % 3 + 1:k % 3 + 1 + N] for k, t in enumerate(whole)]
+    for t, view in zip((g, v, *xs), views):
+        view.copy_(t)
+    a = run_gpu_round(g, v, xs, w, w.start_step, w.H_sel[0],
+                      opts=A.default_opts(pass_=A.PASS_REGISTERS))
+    b = run_gpu_round(views[0], views[1], views[2:], w, w.start_step, w.H_sel[0])
+    assert a["status"] == b["status"] == (A.ERR_NONFINITE if nan else A.OK)
+    bits = {torch.float32: torch.int32, torch.bfloat16: torch.int16}
+    for t, view in zip((g, v, *xs), views):
+        assert torch.equal(t.view(bits[t.dtype]), view.clone().view(bits[t.dtype]))
+    for k, t in enumerate(whole):
+        assert bool((t[:k % 3 + 1] == 3.5).all()) and bool((t[k % 3 + 1 + N:] == 3.5).all())
+    np.testing.assert_allclose(a["drift"], b["drift"], rtol=1e-6)
+    assert np.isnan(b["drift"][0]) == nan and np.isfinite(b["drift"][1:]).all()
+
+
+@pytest.mark.parametrize("form", ["noalloc", "int8_split"])
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+@pytest.mark.parametrize("offset", [1, 2, 3, 5, 7])
+def test_views_at_one_offset_through_the_other_entries(offset, dt, form):
+    """As test_views_at_one_offset_equal_aligned_buffers, through the
+    allocation-free entry point and the split INT8 form."""
+    N = 300_007
+    w = W.small(N, 5, dt, seed=offset)
+    g, v, xs = gpu_inputs(w)
+    whole = [torch.full((offset + N + 9,), 3.5, dtype=t.dtype, device="cuda")
+             for t in (g, v, *xs)]
+    views = [t[offset:offset + N] for t in whole]
+    for t, view in zip((g, v, *xs), views):
+        view.copy_(t)
+    kw = dict(H_sel=w.H_sel[0], H_base=w.H_base, step=w.start_step,
+              schedule=schedule_pair(w.schedule)[0], outer_lr=w.outer_lr,
+              outer_beta=w.outer_beta)
+    if form == "noalloc":
+        run = lambda *bufs: A.sync(*bufs, noalloc=True, **kw)
+    else:
+        run = lambda *bufs: A.sync_int8(*bufs, opts=A.default_opts(pass_=A.PASS_INT8_SPLIT), **kw)
+    a, b = run(g, v, xs), run(views[0], views[1], views[2:])
+    assert a["status"] == b["status"] == A.OK
+    for t, full, view in zip((g, v, *xs), whole, views):
+        assert torch.equal(t, view)
+        assert bool((full[:offset] == 3.5).all()) and bool((full[offset + N:] == 3.5).all())
+    np.testing.assert_allclose(a["drift"], b["drift"], rtol=1e-6)
+
+
 @pytest.mark.parametrize("pass_", [A.PASS_TILE, A.PASS_BULK_COPY], ids=["tile", "bulk_copy"])
 def test_bulk_passes_fall_back_on_unaligned_buffers(pass_):
     """The bulk-copy passes need 16-byte aligned buffers: asked for on a
