@@ -1035,8 +1035,8 @@ static uintptr_t page_locked_gap(uintptr_t p, size_t bytes, bool *one) {
 // slower during the round (bf16 8192^3 matrix products beside 6e7 x 16 bf16
 // 8.7x, beside 1.2e7 x 32 7.4x; 1 GB additions beside the 150M set x 4 bf16
 // 2.0x; 4 MB ones 3 to 14x).  The link needs about 0.6 MB in flight: what
-// kHostInFlight takes, and at least a third of the SMs, which no box was seen
-// to need more than.  Rounds with 152, 64, 48, 38, 28 and 24 blocks: 150M x 4 bf16
+// kHostInFlight takes, and at least a third of the SMs (no GPU measured needs
+// more).  Rounds with 152, 64, 48, 38, 28 and 24 blocks: 150M x 4 bf16
 // (128 bytes a thread) 10.95, 10.94, 10.93, 10.94, 11.26 and 11.00 ms on one GPU,
 // 10.94, 10.94, 10.94, 10.97, 10.95 and 10.96 on another; 5e7 x 12 bf16 7.78, 7.75,
 // 7.75, 7.76, 8.03 and 8.14 ms; 2e7 x 1 fp32 (48 bytes a thread) 1.24, 1.25, 1.25,
