@@ -1006,7 +1006,7 @@ int aloco_int8_decode(const int8_t *codes, const float *scales, size_t N,
 // The first address in [p, p + bytes) that is not page-locked (0: none), p
 // itself being so.  *one stays true where the driver places the range in one
 // allocation: memory locked in several pieces, or whose extent the driver does
-// not tell, is for the copies of the staged round to judge.
+// not tell, is left to the staged round, whose copies check it.
 static uintptr_t page_locked_gap(uintptr_t p, size_t bytes, bool *one) {
     const GetAddressRangeFn fn = address_range_fn();
     for (uintptr_t at = p; at < p + bytes;) {
